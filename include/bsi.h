@@ -271,9 +271,9 @@ bsi_status bsi_geom_rational_init(bsi_geom_rational* g, int64_t X, int64_t Y, in
 bsi_status bsi_field_forward_rational(const bsi_geom_rational* g, const float* phi, float* field,
                                       bsi_stream_t stream);
 
-/* Workspace bytes bsi_field_adjoint_rational needs (partial sums: 6 KB per unit
- * of one z-cell part x one y-cell x a strip of up to 29 x-cells); 0 for an
- * invalid or empty geometry. */
+/* Workspace bytes bsi_field_adjoint_rational needs (partial sums: at most 6 KB
+ * per z-cell x y-cell x strip of up to 29 x-cells); 0 for an invalid or empty
+ * geometry. */
 size_t bsi_rational_adjoint_workspace_bytes(const bsi_geom_rational* g);
 
 /* Transpose of bsi_field_forward_rational (the gradient of a loss with respect

@@ -1,6 +1,6 @@
 """Builds the sm_103a shared library of the package in-tree with nvcc.
 
-Three translation units (C ABI, forward kernels, adjoint kernels) compile in
+The translation units (C ABI and kernels) compile in
 parallel, then link into ``_build/libbsi_gb300.so`` with the CUDA runtime
 linked statically.  ``checked=True`` builds ``libbsi_gb300_checked.so`` with
 BSI_CHECKED defined: every global and shared-memory range a kernel touches is
@@ -19,7 +19,8 @@ ROOT = PKG.parent
 CSRC = PKG / "csrc"
 INCLUDE = ROOT / "include"
 BUILD = PKG / "_build"
-SOURCES = ["bsi_abi.cu", "bsi_forward.cu", "bsi_adjoint.cu", "bsi_probe.cu", "bsi_resample.cu", "bsi_variants.cu", "bsi_rational.cu"]
+SOURCES = ["bsi_abi.cu", "bsi_forward.cu", "bsi_adjoint.cu", "bsi_probe.cu", "bsi_resample.cu", "bsi_variants.cu", "bsi_rational.cu",
+           "bsi_cells_forward.cu", "bsi_cells_adjoint.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -187,6 +187,33 @@ static long long adj_floats(const InstDesc& d) {
     return (f + 3) & ~3LL;  // keep every instance's partials 16-byte aligned
 }
 
+// A volume of integer x-spacing above kMaxSpecializedDx as cells of any width
+// (den = 1, off = 0; bsi_cells.cuh).
+static RatDesc wide_desc(const bsi_geom& g) {
+    RatDesc d;
+    std::memset(&d, 0, sizeof d);
+    d.X = (int)g.X;
+    d.Y = (int)g.Y;
+    d.Z = (int)g.Z;
+    d.num[0] = g.dx;
+    d.num[1] = g.dy;
+    d.num[2] = g.dz;
+    for (int a = 0; a < 3; ++a) d.den[a] = 1;
+    d.nx = (int)g.nx;
+    d.ny = (int)g.ny;
+    d.nz = (int)g.nz;
+    return d;
+}
+
+// Whether a call over n volumes takes those kernels (g: the only volume): their
+// unit is a z-cell or a part of one, whose start is worth it from about 16 rows
+// on (forward + adjoint of 256^3 at 12: 0.405 -> 0.117 ms, at 20: 1.395 -> 0.118
+// ms; 250 x 256 x 200 at (9, 3, 3), 9 rows: 0.093 against 0.113 ms).
+constexpr int kWideMinRows = 16;
+static bool takes_wide(const bsi_geom& g, int n) {
+    return n == 1 && g.dx > kMaxSpecializedDx && g.dy * g.dz >= kWideMinRows && !empty_volume(g);
+}
+
 // Workspace floats an adjoint instance may need: the most (least, with
 // `least`) over every plan the launch may pick -- tile-rows per unit 1, or also
 // kTmaJrows where the volume could take the tensor-copy path, times the table's
@@ -207,6 +234,8 @@ static long long adj_floats_bound(const bsi_geom& g, bool least = false) {
             if (fixed) break;
         }
     }
+    if (!least && takes_wide(g, 1))
+        m = std::max(m, std::max(cell_plan(wide_desc(g), true, false).part_floats, cell_plan(wide_desc(g), true, true).part_floats));
     return m;
 }
 
@@ -546,6 +575,14 @@ static bsi_status forward_impl(const bsi_instance* inst, int n, bsi_dtype dt, cu
     if (dt != BSI_F32 && dt != BSI_BF16) return BSI_ERR_DTYPE;
     bsi_status st = check_instances(inst, n, true, false, dt);
     if (st != BSI_OK) return st;
+    if (n == 1 && dt == BSI_F32 && takes_wide(inst[0].geom, n)) {
+        RatDesc d = wide_desc(inst[0].geom);
+        d.phi = inst[0].phi;
+        d.field = static_cast<float*>(inst[0].field);
+        (void)cudaGetLastError();
+        const cudaError_t e = launch_cells_forward(d, cell_plan(d, false, !misaligned(d.field, 16)), s);
+        return e == cudaSuccess ? BSI_OK : cuda_fail(e);
+    }
     std::vector<InstDesc> all = descs(inst, n, false, dt == BSI_BF16);
     all.erase(std::remove_if(all.begin(), all.end(), [](const InstDesc& d) { return d.units == 0; }), all.end());
     for (const Group& g : plan(all, nullptr)) {
@@ -561,6 +598,20 @@ static bsi_status adjoint_impl(const bsi_instance* inst, int n, void* ws, size_t
                                bool fixed_scratch = false) {
     bsi_status st = check_instances(inst, n, false, true, BSI_F32);
     if (st != BSI_OK) return st;
+    if (n == 1 && takes_wide(inst[0].geom, n)) {
+        const RatDesc d = wide_desc(inst[0].geom);
+        const long long have = (long long)(ws_bytes / sizeof(float));
+        const CellPlan c = cell_plan(d, true, !misaligned(inst[0].grad_field, 16), fixed_scratch ? have : -1);
+        if (!fixed_scratch && adj_floats_bound(inst[0].geom) > have) return BSI_ERR_WORKSPACE;
+        if (c.part_floats <= have) {   // else (fixed scratch): the plans below have smaller ones
+            if (!ws) return BSI_ERR_WORKSPACE;
+            if (misaligned(ws, 16)) return BSI_ERR_ALIGN;
+            (void)cudaGetLastError();
+            const cudaError_t e =
+                launch_cells_adjoint(d, c, inst[0].grad_field, inst[0].grad_phi, static_cast<float*>(ws), s);
+            return e == cudaSuccess ? BSI_OK : cuda_fail(e);
+        }
+    }
     long long ws_floats = 0;
     const bool tma = tensor_map_encoder() != nullptr;
     const std::vector<Group> groups =
@@ -662,6 +713,106 @@ static void check_forward_tma(const InstDesc& d0, bool bf16, int c, RangeChecker
         if (u.x0 + d.gcells * d.dx < d.X && u.nvox != d.gcells * d.dx) rc.fail("box past its strip", u.x0, u.nvox);
         if (u.ncell > d.gcells || (long long)(u.ncell - 1) * tile + tile > rowb) rc.fail("lane past block row", u.ncell, rowb);
     }
+}
+
+// The kernels on cells of any width: strips and lane runs tile every row once and
+// fit a staged row, blocks and weights fit the warp's shared memory, units tile
+// the planes and rows, grid reads stay in the grid, and the reduce reads only
+// partial sums that a unit writes.
+static void check_cells(const RatDesc& d, const CellPlan& c, bool adjoint, RangeChecker& rc, bool cover) {
+    if (c.parts < 1 || c.run < 1 || c.run > (c.parts == 1 ? kCellRunMax : kCellWideRun)) rc.fail("cell parts", c.parts, c.run);
+    if (c.parts * c.sc > kLanes || c.nc > kLanes || c.nc != c.sc + kHalo) rc.fail("strip cells", c.sc, c.parts);
+    const int budget = kCellWarpBudget;
+    if (c.warp_bytes > budget || c.warp_bytes % 128 != 0 || c.head_bytes % 128 != 0) rc.fail("warp shared memory", c.warp_bytes, budget);
+    if (c.head_bytes < kCellWeightOff + 16 * (c.ymax + c.zmax) || c.head_bytes + kCellStages * c.stage_bytes > c.warp_bytes ||
+        c.rb < 1 || c.rb > kLanes || c.rb * c.slot > c.stage_bytes || c.slot % 16 != 0)
+        rc.fail("ring layout", c.rb, c.slot);
+    // spare run: RUN voxels and a row's phase
+    if (c.vec && (c.run != 4 || d.X % 4 || d.num[0] % 4)) rc.fail("vector runs", c.run, d.X);
+    if (kCellSpareOff + 12 * c.run + 12 > kCellWeightOff || 8 * kCellStages > kCellSpareOff) rc.fail("spare run", c.run, kCellWeightOff);
+    if (c.parts == 1 && (long long)c.nsx * c.sc < c.ncx) rc.fail("strips", c.nsx, c.sc);
+    int x = 0;
+    for (int xs = 0; xs < c.nsx; ++xs) {
+        const CellStrip s = cell_strip(d, c, xs);
+        if (s.cells < 1 || s.sx0 != x || s.sx1 <= s.sx0) rc.fail("strip start", s.sx0, x);
+        if (12 * (s.sx1 - s.sx0) + 30 > c.slot) rc.fail("staged row overflow", s.sx1 - s.sx0, c.slot);
+        if (s.c0 + s.cells + kHalo > d.nx) rc.fail("grid columns", s.c0 + s.cells + kHalo, d.nx);
+        for (int lane = 0; lane < kLanes; ++lane) {
+            const CellRun r = cell_run(d, c, s, lane);
+            if (r.cnt < 0 || r.cnt > c.run) rc.fail("lane run", r.cnt, c.run);
+            if (r.cnt == 0) continue;
+            if (c.vec && (r.cnt != 4 || r.xa % 4)) rc.fail("vector run", r.xa, r.cnt);
+            if (r.xa != x) rc.fail("lane run start", r.xa, x);
+            for (int i = 0; i < r.cnt; ++i) {
+                const long long q = (long long)(r.xa + i) * d.den[0] + d.off[0];
+                if (q / d.num[0] != r.col) rc.fail("voxel in another cell", r.xa + i, r.col);
+            }
+            // every unpredicated access of a regular strip (run - 1 voxels, a row's phase) stays in the staged row
+            if (r.cnt >= c.run - 1 && 12 * (r.xa - s.sx0 + c.run - 1) + 15 > c.slot) rc.fail("lane past staged row", r.xa, c.slot);
+            x += r.cnt;
+        }
+        if (x != s.sx1) rc.fail("strip end", x, s.sx1);
+    }
+    if (x != d.X) rc.fail("row not covered", x, d.X);
+    if (!cover) return;
+    std::vector<unsigned char> plane((size_t)d.Y * d.Z, 0), written(adjoint ? (size_t)(c.part_floats / 3) : 0, 0);
+    for (long long un = 0; un < c.units; ++un) {
+        const CellUnit u = cell_unit(d, c, un);
+        if (u.y1 <= u.y0 || u.y1 - u.y0 > c.ymax || u.z1 < u.z0 || u.z1 - u.z0 > c.zmax || u.y1 > d.Y || u.z1 > d.Z ||
+            u.y0 < 0 || u.z0 < 0)
+            rc.fail("unit rows and planes", u.y1 - u.y0, u.z1 - u.z0);
+        if (u.jy + 4 > d.ny || u.kz1 + kHalo > d.nz || u.kz1 <= u.kz0 || u.kz1 - u.kz0 > c.zc) rc.fail("unit cells", u.jy, u.kz0);
+        for (int z = u.z0; z < u.z1; ++z) {
+            const int kz = (int)(((long long)z * d.den[2] + d.off[2]) / d.num[2]);
+            if (kz < u.kz0 || kz >= u.kz1) rc.fail("plane in another cell", z, kz);
+            for (int y = u.y0; y < u.y1; ++y) {
+                if (((long long)y * d.den[1] + d.off[1]) / d.num[1] != u.jy) rc.fail("row in another cell", y, u.jy);
+                if (u.xs == 0) plane[(size_t)z * d.Y + y]++;
+            }
+        }
+        if (!adjoint) continue;
+        for (int pz = 0; pz < u.kz1 - u.kz0 + kHalo; ++pz)
+            for (int m = 0; m < 4; ++m)
+                for (int j = 0; j < c.nc; ++j) {
+                    const long long e = cell_part(c, un, pz, m, j);
+                    if (e < 0 || e + 3 > c.part_floats) rc.fail("partial write", e, c.part_floats);
+                    else written[(size_t)(e / 3)]++;
+                }
+    }
+    for (size_t i = 0; i < plane.size(); ++i)
+        if (plane[i] != 1) {
+            rc.fail("row taken != once", (long long)i, plane[i]);
+            break;
+        }
+    if (!adjoint) return;
+    std::vector<unsigned char> read(written.size(), 0);
+    for (int gz = 0; gz < d.nz; ++gz)
+        for (int gy = 0; gy < d.ny; ++gy)
+            for (int gx = 0; gx < d.nx; ++gx) {
+                const int zdiv = c.zsplit > 1 ? c.zsplit : 1, nch = c.zsplit > 1 ? c.ncz : c.nzu;
+                for (int ch = imin(nch - 1, gz / c.zc); ch >= 0; --ch) {
+                    const int pz = gz - ch * c.zc;
+                    if (pz >= imin(c.zc, c.ncz - ch * c.zc) + kHalo) break;
+                    for (int zi = ch * zdiv; zi < (ch + 1) * zdiv; ++zi)
+                        for (int xs = imin(c.nsx - 1, gx / c.sc); xs >= 0; --xs) {
+                            const int j = gx - xs * c.sc;
+                            if (j >= imin(c.sc, c.ncx - xs * c.sc) + kHalo) break;
+                            for (int m = 0; m < 4; ++m) {
+                                const int jy = gy - m;
+                                if (jy < 0 || jy >= c.ncy) continue;
+                                const long long e = cell_part(c, ((long long)zi * c.ncy + jy) * c.nsx + xs, pz, m, j);
+                                if (e < 0 || e + 3 > c.part_floats || !written[(size_t)(e / 3)]) rc.fail("partial read", e, c.part_floats);
+                                else read[(size_t)(e / 3)]++;
+                            }
+                        }
+                }
+            }
+    // every column of a cell's sums reaches one control point (columns past a short strip hold zeros)
+    for (size_t i = 0; i < read.size(); ++i)
+        if (read[i] > 1) {
+            rc.fail("partial read twice", (long long)i, read[i]);
+            break;
+        }
 }
 
 static void check_forward_group(const Group& g, int ob, RangeChecker& rc, bool cover) {
@@ -996,15 +1147,18 @@ bsi_status bsi_get_tile_config(int32_t dx, int32_t dy, int32_t dz, bsi_tile_conf
 
 bsi_status bsi_check_device_status(bsi_stream_t stream, uint32_t* flags) {
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    static thread_local unsigned words[5];
+    static thread_local unsigned words[7];
     cudaError_t e = forward_err_read_clear(&words[0], s);
     if (e == cudaSuccess) e = adjoint_err_read_clear(&words[1], s);
     if (e == cudaSuccess) e = resample_err_read_clear(&words[2], s);
     if (e == cudaSuccess) e = variants_err_read_clear(&words[3], s);
     if (e == cudaSuccess) e = rational_err_read_clear(&words[4], s);
+    if (e == cudaSuccess) e = cells_forward_err_read_clear(&words[5], s);
+    if (e == cudaSuccess) e = cells_adjoint_err_read_clear(&words[6], s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e);
-    const uint32_t w = words[0] | words[1] | words[2] | words[3] | words[4];
+    uint32_t w = 0;
+    for (const unsigned x : words) w |= x;
     if (flags) *flags = w;
     return w ? BSI_ERR_DEVICE_STATUS : BSI_OK;
 }
@@ -1122,9 +1276,23 @@ bsi_status bsi_field_forward_rational(const bsi_geom_rational* g, const float* p
     return e == cudaSuccess ? BSI_OK : cuda_fail(e);
 }
 
+// Workspace floats of the adjoint: 4 rows x 32 columns x 3 channels per grid
+// plane of units of zc z-cells x one y-cell x up to 29 x-cells (232 voxels); the
+// launch picks a plan of at most this many partial sums (or its smallest).
+static long long rational_part_floats(const RatDesc& d) {
+    auto cells = [&](int a, int N) { return cdiv((long long)(N - 1) * d.den[a] + d.off[a] + 1, d.num[a]); };
+    auto widest = [&](int a) { return (d.num[a] + d.den[a] - 1) / d.den[a]; };
+    const long long ncz = cells(2, d.Z);
+    const long long strips = cells(1, d.Y) * cdiv(cells(0, d.X), imin(kGroupCells, 232 / widest(0)));
+    int zc = 4;
+    while (zc > 1 && (cdiv(ncz, zc) * strips < 6000 || zc * widest(2) > kCellRowsMax)) zc /= 2;
+    const long long f = cdiv(ncz, zc) * strips * (zc + kHalo) * 4 * kLanes * 3;
+    return std::max(f, std::max(cell_plan(d, true, false, f).part_floats, cell_plan(d, true, true, f).part_floats));
+}
+
 size_t bsi_rational_adjoint_workspace_bytes(const bsi_geom_rational* g) {
     if (check_rational(g) != BSI_OK || g->X == 0 || g->Y == 0 || g->Z == 0) return 0;
-    return (size_t)rational_adjoint_plan(rat_desc(*g)).part_floats * sizeof(float);
+    return (size_t)rational_part_floats(rat_desc(*g)) * sizeof(float);
 }
 
 bsi_status bsi_field_adjoint_rational(const bsi_geom_rational* g, const float* grad_field, float* grad_phi,
@@ -1142,11 +1310,13 @@ bsi_status bsi_field_adjoint_rational(const bsi_geom_rational* g, const float* g
     if (!grad_field) return BSI_ERR_NULL;
     if (misaligned(grad_field, 4)) return BSI_ERR_ALIGN;
     const RatDesc d = rat_desc(*g);
-    const size_t need = (size_t)rational_adjoint_plan(d).part_floats * sizeof(float);
+    const long long floats = rational_part_floats(d);
+    const size_t need = (size_t)floats * sizeof(float);
     if (!workspace || workspace_bytes < need) return BSI_ERR_WORKSPACE;
     if (misaligned(workspace, 16)) return BSI_ERR_ALIGN;
     (void)cudaGetLastError();
-    const cudaError_t e = launch_adjoint_rational(d, grad_field, grad_phi, static_cast<float*>(workspace), s);
+    const cudaError_t e =
+        launch_cells_adjoint(d, cell_plan(d, true, !misaligned(grad_field, 16), floats), grad_field, grad_phi, static_cast<float*>(workspace), s);
     return e == cudaSuccess ? BSI_OK : cuda_fail(e);
 }
 
@@ -1218,6 +1388,15 @@ int bsi_selfcheck_ranges(const bsi_instance* inst, int n, int op, int cover, cha
         for (int i = 0; i < n; ++i) ok = ok && check_geom(&inst[i].geom) == BSI_OK;
         if (!ok) {
             rc.fail("invalid geometry", n, 0);
+        } else if ((op == 0 || op == 2) && n == 1 && takes_wide(inst[0].geom, n)) {
+            // cells of any width, for aligned and unaligned arrays, and within the least no-alloc plan
+            const RatDesc d = wide_desc(inst[0].geom);
+            const long long bound = adj_floats_bound(inst[0].geom);
+            for (int vec = 0; vec < 2; ++vec) {
+                const CellPlan c = cell_plan(d, op == 2, vec != 0);
+                check_cells(d, c, op == 2, rc, cover != 0);
+                if (c.part_floats > bound) rc.fail("planned workspace over the documented bound", c.part_floats, bound);
+            }
         } else if (op != 2) {
             std::vector<InstDesc> all = descs(inst, n, false, op == 1 || op == 6);
             all.erase(std::remove_if(all.begin(), all.end(), [](const InstDesc& d) { return d.units == 0; }),

@@ -320,6 +320,204 @@ BSI_HD long long rational_dim(long long N, int num, int den, int off) {
     return N > 0 ? ((N - 1) * den + off) / num + 4 : 4;
 }
 
+// Cells of any width (bsi_cells.cu: non-integer spacing, and integer x-spacings
+// above kMaxSpecializedDx as den = 1, off = 0).  A cell of an axis holds the
+// voxels x with floor((x den + off) / num) = its index; its width is the floor
+// or the ceiling of num / den, less at the volume's ends.  A warp takes strips
+// of sc x-cells.  A cell of up to 7 voxels belongs to one lane; a wider one is
+// shared by `parts` neighbouring lanes, each taking an even run of it (floor or
+// ceiling of width / parts, at most 7: odd runs keep the 12-byte voxel stride
+// of the lanes off common shared-memory banks), so that a row's work is spread
+// over the whole warp at every spacing.
+constexpr int kCellRunMax = 7;      // cells of up to this many voxels belong to one lane
+constexpr int kCellWideRun = 7;     // run bound for wider cells
+constexpr int kCellRowsMax = 64;    // rows (planes) of a y-cell (z-cell): spacing <= 64
+
+// First voxel of cell k of an axis: the least x with x den + off >= k num (k up
+// to a strip past the last cell: k num stays below 2^30 + 2^22, see the limits of
+// the API).
+BSI_HD int cell_first(int k, int num, int den, int off) {
+    const int t = k * num - off;
+    return t <= 0 ? 0 : den == 1 ? t : (int)((unsigned)(t + den - 1) / (unsigned)den);
+}
+
+struct CellPlan {
+    int ncx, ncy, ncz;   // cells per axis
+    int parts, run;      // lanes per x-cell, and the longest run of one lane
+    int vec;             // runs of 4 voxels on 16-byte boundaries (see cell_plan)
+    int sc, nsx;         // x-cells per strip, strips
+    int nc;              // columns a strip touches: sc + 3
+    int zc, zsplit;      // z-cells per unit, or (zsplit > 1, zc = 1) units per z-cell
+    int nzu;             // z-units: ceil(ncz / zc) or ncz zsplit
+    int ymax, zmax;      // most rows of a unit, most planes
+    int slot;            // bytes of one staged row (16-byte multiple)
+    int rb;              // rows per block
+    int stage_bytes;     // rb slots
+    int head_bytes;      // per warp, ahead of the ring: barriers, a spare row, the unit's y and z weights
+    int warp_bytes;
+    long long units;
+    long long part_floats;   // adjoint: partial sums
+};
+
+constexpr int kCellSpareOff = 64;    // spare run (adjoint: zeros; forward: never stored) after the barriers
+constexpr int kCellWeightOff = 192;  // y weights, then z weights (16 bytes each)
+constexpr int kCellStages = 2;       // blocks in flight per warp
+
+// One unit: planes [z0, z1) of the z-cells [kz0, kz1), rows [y0, y1) of y-cell
+// jy, x-cells [c0, c0 + cells) with voxels [sx0, sx1).
+struct CellUnit {
+    int xs, jy, kz0, kz1, z0, z1, y0, y1;
+};
+
+BSI_HD CellUnit cell_unit(const RatDesc& d, const CellPlan& c, long long un) {
+    CellUnit u;
+    int zi;
+    if (c.units <= 0x7fffffffLL) {   // 32-bit division (64-bit division is a long sequence)
+        const unsigned t = (unsigned)un / (unsigned)c.nsx;
+        u.xs = (int)((unsigned)un - t * (unsigned)c.nsx);
+        zi = (int)(t / (unsigned)c.ncy);
+        u.jy = (int)(t - (unsigned)zi * (unsigned)c.ncy);
+    } else {
+        u.xs = (int)(un % c.nsx);
+        const long long t = un / c.nsx;
+        u.jy = (int)(t % c.ncy);
+        zi = (int)(t / c.ncy);
+    }
+    if (c.zsplit > 1) {
+        u.kz0 = zi / c.zsplit;
+        u.kz1 = u.kz0 + 1;
+    } else {
+        u.kz0 = zi * c.zc;
+        u.kz1 = imin(u.kz0 + c.zc, c.ncz);
+    }
+    u.z0 = cell_first(u.kz0, d.num[2], d.den[2], d.off[2]);
+    u.z1 = imin(d.Z, cell_first(u.kz1, d.num[2], d.den[2], d.off[2]));
+    if (c.zsplit > 1) {
+        const int n = u.z1 - u.z0, p = zi - u.kz0 * c.zsplit, a = u.z0;
+        u.z0 = a + n * p / c.zsplit;
+        u.z1 = a + n * (p + 1) / c.zsplit;
+    }
+    u.y0 = cell_first(u.jy, d.num[1], d.den[1], d.off[1]);
+    u.y1 = imin(d.Y, cell_first(u.jy + 1, d.num[1], d.den[1], d.off[1]));
+    return u;
+}
+
+// The x side of strip xs and of one lane in it: its part lp of cell c0 + lc.
+struct CellStrip {
+    int c0, cells, sx0, sx1;
+};
+struct CellRun {
+    int col, xa, cnt;   // the lane's cell, first voxel and voxels (0: none)
+};
+
+BSI_HD CellStrip cell_strip(const RatDesc& d, const CellPlan& c, int xs) {
+    CellStrip s;
+    s.c0 = xs * c.sc;
+    s.cells = imin(c.sc, c.ncx - s.c0);
+    s.sx0 = cell_first(s.c0, d.num[0], d.den[0], d.off[0]);
+    s.sx1 = imin(d.X, cell_first(s.c0 + s.cells, d.num[0], d.den[0], d.off[0]));
+    return s;
+}
+
+BSI_HD CellRun cell_run(const RatDesc& d, const CellPlan& c, const CellStrip& s, int lane) {
+    CellRun r;
+    const int lc = lane / c.parts, lp = lane - lc * c.parts;
+    r.col = s.c0 + lc;
+    r.xa = s.sx0;
+    r.cnt = 0;
+    if (lc < s.cells) {
+        const int a = cell_first(r.col, d.num[0], d.den[0], d.off[0]);
+        const int w = imin(d.X, cell_first(r.col + 1, d.num[0], d.den[0], d.off[0])) - a;
+        const int i0 = c.vec ? imin(w, 4 * lp) : w * lp / c.parts;
+        const int i1 = c.vec ? imin(w, 4 * lp + 4) : w * (lp + 1) / c.parts;
+        r.xa = a + i0;
+        r.cnt = i1 - i0;
+    }
+    return r;
+}
+
+// Float offset of a unit's partial sums: plane pz (0 .. zc + 2), grid row m (0 ..
+// 3), column j (0 .. nc - 1).
+BSI_HD long long cell_part(const CellPlan& c, long long un, int pz, int m, int j) {
+    return ((un * (c.zc + kHalo) + pz) * 4 + m) * (3LL * c.nc) + 3LL * j;
+}
+
+// Shared memory of one warp: twelve warps (three CTAs) share an SM's 228 KB,
+// 1 KB per CTA set aside.
+constexpr int kCellWarpsPerSm = 12;
+constexpr int kCellWarpBudget = (225 * 1024 / kCellWarpsPerSm) & ~127;
+
+// Plan of a volume (a rule of its geometry only, so that a workspace query
+// needs no device).  Adjoint: z-cells per unit, or units per z-cell (forward:
+// one cell, or a part of it), by a cost model of rounds over the warps of a
+// 152-SM GPU x rows of a unit, in units of one staged row; a last, partial
+// round costs 0.6 + 0.4 x its fill (a lone warp per scheduler runs faster); a unit costs about kUnitRows rows to start and half
+// a row per plane of partial sums, and a partial sum is written and read once.  Only plans of
+// at most max_floats partial sums (when >= 0); if none fits, the smallest.
+// vec: rows on 16-byte boundaries (X % 4 == 0, aligned array) may take runs of
+// exactly 4 voxels -- three 16-byte vectors at a lane stride of 48 bytes, which
+// meets no bank conflict -- where the x-spacing is an integer multiple of 4 above
+// kCellRunMax.
+inline CellPlan cell_plan(const RatDesc& d, bool adjoint, bool vec, long long max_floats = -1) {
+    constexpr double kUnitRows = 4.0;
+    CellPlan c = {};
+    auto cells = [&](int a, int N) { return (int)(((long long)(N - 1) * d.den[a] + d.off[a]) / d.num[a]) + 1; };
+    auto widest = [&](int a, int N) { return imin(N, (d.num[a] + d.den[a] - 1) / d.den[a]); };
+    c.ncx = cells(0, d.X);
+    c.ncy = cells(1, d.Y);
+    c.ncz = cells(2, d.Z);
+    const int w = (d.num[0] + d.den[0] - 1) / d.den[0];
+    c.vec = vec && d.X % 4 == 0 && d.den[0] == 1 && d.off[0] == 0 && w % 4 == 0 && w > kCellRunMax;
+    c.parts = w <= kCellRunMax ? 1 : c.vec ? w / 4 : (w + kCellWideRun - 1) / kCellWideRun;
+    c.run = (w + c.parts - 1) / c.parts;
+    const int per = c.parts == 1 ? kGroupCells : kLanes / c.parts;
+    c.nsx = (int)cdiv(c.ncx, per);
+    c.sc = (int)cdiv(c.ncx, c.nsx);   // strips of even width
+    c.nsx = (int)cdiv(c.ncx, c.sc);
+    c.nc = c.sc + kHalo;
+    const int vox = imin(d.X, (int)((long long)c.sc * d.num[0] / d.den[0]) + 1);
+    c.slot = (12 * vox + 32 + 15) & ~15;
+    c.ymax = widest(1, d.Y);
+    c.zmax = kCellRowsMax;
+    const int zw = widest(2, d.Z);
+    const double rows = (double)d.num[1] / d.den[1], planes = (double)d.num[2] / d.den[2];
+    const double slots = 152.0 * kCellWarpsPerSm;
+    c.zc = c.zsplit = 1;
+    auto size = [&](CellPlan& p) {
+        p.nzu = p.zsplit > 1 ? p.ncz * p.zsplit : (int)cdiv(p.ncz, p.zc);
+        p.units = (long long)p.nzu * p.ncy * p.nsx;
+        p.part_floats = adjoint ? p.units * (p.zc + kHalo) * 4 * 3 * p.nc : 0;
+    };
+    CellPlan best = c, p = c;
+    double best_t = -1;
+    bool fits = false;
+    for (int k = adjoint ? 0 : 7; k < 14; ++k) {   // zc = 8 .. 1, then 2, 4 .. 64 units per z-cell
+        p.zc = k < 8 ? 8 - k : 1;
+        p.zsplit = k < 8 ? 1 : 1 << (k - 7);
+        if (p.zc * zw > kCellRowsMax || p.zsplit > zw) continue;
+        size(p);
+        const bool f = max_floats < 0 || p.part_floats <= max_floats;
+        const double n = p.units / slots, full = (double)(long long)n, part = n - full;
+        const double start = adjoint ? kUnitRows + 0.5 * (p.zc + kHalo) : kUnitRows;
+        const double t = (full + (part > 1e-9 ? 0.6 + 0.4 * part : 0.0)) * (planes * p.zc / p.zsplit * rows + start) +
+                         p.part_floats * 4.0 / (12.0 * vox * slots);
+        if (best_t < 0 || (f && !fits) || (f == fits && (f ? t < best_t : p.part_floats < best.part_floats))) {
+            best = p;
+            best_t = t;
+            fits = f;
+        }
+    }
+    c = best;
+    c.zmax = imin(kCellRowsMax, c.zc * zw);
+    c.head_bytes = pad128(kCellWeightOff + 16 * (c.ymax + c.zmax));
+    int rb = (kCellWarpBudget - c.head_bytes) / (kCellStages * c.slot);
+    rb = imax(1, imin(imin(rb, c.ymax), kLanes));
+    c.rb = (int)cdiv(c.ymax, cdiv(c.ymax, rb));   // even blocks
+    c.stage_bytes = c.rb * c.slot;
+    c.warp_bytes = pad128(c.head_bytes + kCellStages * c.stage_bytes);
+    return c;
+}
+
 constexpr int kMaxWarpsPerCta = 8;
 constexpr int kAdjWarpsMax = 4;   // adjoint partials kernel: 4-warp CTAs (register budget)
 constexpr int kSmemBudget = 200 * 1024;   // dynamic shared memory per CTA we allow

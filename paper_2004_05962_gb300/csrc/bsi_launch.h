@@ -15,10 +15,10 @@ namespace bsi {
 // for that grid's completion before touching memory.  After a kernel that never
 // signals, this is an ordinary launch.
 template <typename... P, typename... A>
-cudaError_t launch_pdl(void (*kern)(P...), int grid, int threads, int smem, cudaStream_t s, A&&... args) {
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 threads, int smem, cudaStream_t s, A&&... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
+    cfg.gridDim = grid;
+    cfg.blockDim = threads;
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -46,17 +46,16 @@ cudaError_t launch_forward_tile_variant(const Batch<1>& b, bool lerp, cudaStream
 cudaError_t variants_err_read_clear(unsigned* out, cudaStream_t s);
 
 // Non-integer, non-aligned spacing (bsi_rational.cu).
-int rational_warps_per_cta(int nx);
 cudaError_t launch_forward_rational(const RatDesc& d, cudaStream_t s, LaunchInfo* info);
-// Adjoint of the non-integer-spacing path: its unit counts and partial-sum
-// floats (the workspace), and its two launches (partials, reduce).
-struct RatAdjPlan {
-    int ncx, ncy, ncz, nsx, sc, zc;   // cells per axis, strips, cells per strip, z-cells per unit
-    long long part_floats;
-};
-RatAdjPlan rational_adjoint_plan(const RatDesc& d);
-cudaError_t launch_adjoint_rational(const RatDesc& d, const float* grad, float* dphi, float* part, cudaStream_t s);
 cudaError_t rational_err_read_clear(unsigned* out, cudaStream_t s);
+
+// Cells of any width (bsi_cells_forward.cu, bsi_cells_adjoint.cu): c from
+// cell_plan(d, adjoint).
+cudaError_t launch_cells_forward(const RatDesc& d, const CellPlan& c, cudaStream_t s);
+cudaError_t launch_cells_adjoint(const RatDesc& d, const CellPlan& c, const float* grad, float* dphi, float* part,
+                                 cudaStream_t s);
+cudaError_t cells_forward_err_read_clear(unsigned* out, cudaStream_t s);
+cudaError_t cells_adjoint_err_read_clear(unsigned* out, cudaStream_t s);
 
 // Forward of one volume on the tensor-store path (fwd_tma_rows gives rb > 0;
 // map: the output as a 3-D tensor of 8-byte elements, box (strip, rb, 1));
