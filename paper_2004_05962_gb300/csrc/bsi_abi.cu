@@ -150,6 +150,7 @@ static void fill_desc(InstDesc& d, const bsi_geom& g, bool adjoint, bool bf16 = 
     } else {
         d.zchunk = zchunk;
         d.tma_rows = tma_block_rows(d.dx, d.dy);
+        d.row_block = row_block_rows(d.dx, d.dy);
         d.nxg = empty ? 0 : (int)cdiv(d.nx, kGroupCells);
         d.nzc = empty ? 0 : (int)cdiv(d.ncz, zchunk);
         d.units = (long long)d.nzc * d.ncyu * d.nxg;
@@ -386,10 +387,10 @@ static std::vector<Group> plan(const std::vector<InstDesc>& all, long long* ws_f
 }
 
 template <int MAXB>
-static void to_batch(const Group& g, Batch<MAXB>& b) {
+static void to_batch(const Group& g, Batch<MAXB>& b, bool adjoint = false) {
     std::memset(&b, 0, sizeof b);
     b.n = (int)g.inst.size();
-    b.buf_bytes = g.tma ? g.tma_stage : stage_buf_bytes(g.dxmax);
+    b.buf_bytes = g.tma ? g.tma_stage : adjoint ? row_stage_bytes(g.dxmax) : stage_buf_bytes(g.dxmax);
     b.stages = g.tma ? tma_default_stages(g.tma_stage) : 0;
     b.warps_req = g.tma ? 0 : g.warps_req;
     for (int i = 0; i < b.n; ++i) {
@@ -490,7 +491,7 @@ static cudaError_t run_group(const Group& g, Op op, bool bf16, float* part, long
     (void)cudaGetLastError();  // a launch must not report an earlier call's returned error
     if (g.inst.size() == 1) {
         Batch<1> b;
-        to_batch(g, b);
+        to_batch(g, b, op != Op::Forward);
         if (op == Op::Forward) {
             if (bf16_odd_strips(b.inst[0], bf16, g.generic)) b.total_units = b.inst[0].units;
             const int rb = forward_tma_rows(b.inst[0], bf16, g.generic);
@@ -511,7 +512,7 @@ static cudaError_t run_group(const Group& g, Op op, bool bf16, float* part, long
         return launch_adjoint_reduce(b, part, ws_floats, s, nullptr);
     }
     static thread_local Batch<kMaxBatch> b;  // ~9 KB: kept off the stack
-    to_batch(g, b);
+    to_batch(g, b, op != Op::Forward);
     if (op == Op::Forward) return launch_forward(b, bf16, g.generic, s, nullptr);
     if (op == Op::AdjointPartials) {
         if (g.tma) {
@@ -859,7 +860,6 @@ static void check_forward_group(const Group& g, int ob, RangeChecker& rc, bool c
 }
 
 static void check_adjoint_group(const Group& g, long long ws_floats, RangeChecker& rc, bool cover) {
-    const int buf = stage_buf_bytes(g.dxmax);
     std::vector<unsigned char> written(cover ? (size_t)(ws_floats / 3 + 1) : 0, 0);
     for (const InstDesc& d : g.inst) {
         const long long field_elems = 3LL * d.X * d.Y * d.Z;
@@ -891,32 +891,30 @@ static void check_adjoint_group(const Group& g, long long ws_floats, RangeChecke
                 if (st < kTmaMinStages || st > kTmaMaxStages || (long long)w * tma_warp_smem(tsb, st) + 128 > kTmaSmemBudget)
                     rc.fail("tensor-copy shared memory over budget", w, tsb);
             }
-            // a bulk load covers the 16-byte-aligned superset of the row: <= nbytes + 30
-            if (!g.tma && 30 + u.nvox * 12 > buf) rc.fail("staging overflow", u.nvox, buf);
-            // unpredicated reads of a specialised spacing: every lane reads dx voxels,
-            // inside [0, nvox) or, in a ragged unit, the zeros [nvox, nvox + zv)
+            // row-copy path: a bulk load covers the 16-byte-aligned superset of the row, <=
+            // nbytes + 30; a block's rows fit the stage, the twelve warps' rings the SM
+            const int slot = stage_buf_bytes(d.dx), stage = row_stage_bytes(g.dxmax);
+            if (!g.tma && 30 + u.nvox * 12 > slot) rc.fail("staging overflow", u.nvox, slot);
+            if (!g.tma && (d.row_block < 1 || d.row_block > kLanes || d.row_block * slot > stage))
+                rc.fail("row block over stage", d.row_block, slot);
+            if (!g.tma && stage % 16 != 0) rc.fail("stage alignment", stage, 16);
             const bool spec = d.dx <= kMaxSpecializedDx && !g.generic && !g.tma;
-            bool ragged = false;
-            for (int lane = 0; lane < kLanes; ++lane) {
-                const int cell = u.col0 - kHalo + lane;
-                const int nv = (cell >= 0 && cell < d.ncx) ? imin(d.dx, d.X - cell * d.dx) : 0;
-                ragged = ragged || nv != d.dx;
-            }
-            const int zv = imin(d.dx, kLanes * d.dx - u.nvox);
-            if (spec && ragged && 15 + 12 * (u.nvox + zv) > buf) rc.fail("zeroed tail overflow", u.nvox + zv, buf);
-            if (!g.tma && warps_per_cta(adj_warp_smem(buf)) * adj_warp_smem(buf) > kSmemBudget)
-                rc.fail("adjoint shared memory over budget", buf, kSmemBudget);
+            if (spec && kRowSpareOff + 16 * ((3 * d.dx + 6) / 4) > kRowHeadBytes) rc.fail("spare zeros", d.dx, kRowHeadBytes);
+            const int req = kAdjWarpsMax;
+            if (!g.tma && warps_per_cta(adj_warp_smem(stage), req) * adj_warp_smem(stage) > kSmemBudget)
+                rc.fail("adjoint shared memory over budget", stage, kSmemBudget);
             for (int lane = 0; lane < kLanes; ++lane) {
                 const int cell = u.col0 - kHalo + lane;
                 const int nv = (cell >= 0 && cell < d.ncx) ? imin(d.dx, d.X - cell * d.dx) : 0;
                 const int xl = cell * d.dx - u.xs;
                 if (nv > 0 && (xl < 0 || xl + nv > u.nvox)) rc.fail("lane voxels outside strip", xl, u.nvox);
-                if (spec) {
-                    const int rl = nv == 0 ? u.nvox : xl;   // the kernel's read start
-                    if (rl < 0 || rl + d.dx > (ragged ? u.nvox + zv : u.nvox))
-                        rc.fail("unpredicated read outside row and zeros", rl, u.nvox);
-                    if (nv > 0 && nv < d.dx && xl + nv != u.nvox)   // its missing voxels are the zeros
-                        rc.fail("cut tile does not end at the row end", xl + nv, u.nvox);
+                if (spec && nv > 0) {
+                    // unpredicated reads of a specialised spacing: inside [0, nvox), or (a cut tile,
+                    // the last of its row) the zeros after it; vector reads end with the 16-byte
+                    // group of the tile's last float
+                    if (nv < d.dx && (xl + nv != u.nvox || d.dx - nv > d.dx - 1)) rc.fail("cut tile does not end at the row end", xl + nv, u.nvox);
+                    if (12 * (xl + d.dx) + 15 > slot) rc.fail("tile past its staged row", xl, slot);
+                    if (nv < d.dx && 15 + 12 * u.nvox + 12 * (d.dx - 1) > slot) rc.fail("zeroed tail overflow", u.nvox, slot);
                 }
                 const int j = lane - kHalo;
                 if (j < 0 || u.col0 + j >= d.nx) continue;

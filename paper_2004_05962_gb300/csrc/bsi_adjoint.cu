@@ -27,7 +27,9 @@ __global__ void __launch_bounds__(kAdjMaxWarps * kLanes, 3)
     const int warp = threadIdx.x >> 5;
     unsigned char* wsm = smem + (size_t)warp * adj_warp_smem(b.buf_bytes);
     uint64_t* bars = reinterpret_cast<uint64_t*>(wsm);           // mbarrier of stage s: bars[s]
-    unsigned char* bufs = wsm + 16 * kLoadStages;                 // kLoadStages ring buffers
+    const uint32_t spare = smem_u32(wsm + kRowSpareOff);          // zeros: empty tiles read them
+    unsigned char* ring = wsm + kRowHeadBytes;                    // kLoadStages stages
+    sts_f32(spare + 4u * lane, 0.f);
     if (lane == 0) {
         for (int s = 0; s < kLoadStages; ++s) mbar_init(bars + s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -45,17 +47,17 @@ __global__ void __launch_bounds__(kAdjMaxWarps * kLanes, 3)
         const long long ul = uu - d.unit_begin;
         bool ok;
         if (GENERIC) {
-            ok = adjoint_unit<0>(d, ul, bars, bufs, b.buf_bytes, lane, q, part, ws_floats, &g_err);
+            ok = adjoint_unit<0>(d, ul, bars, spare, ring, b.buf_bytes, lane, q, part, ws_floats, &g_err);
         } else {
             switch (d.dx) {
-                case 1: ok = adjoint_unit<1>(d, ul, bars, bufs, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
-                case 2: ok = adjoint_unit<2>(d, ul, bars, bufs, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
-                case 3: ok = adjoint_unit<3>(d, ul, bars, bufs, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
-                case 4: ok = adjoint_unit<4>(d, ul, bars, bufs, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
-                case 5: ok = adjoint_unit<5>(d, ul, bars, bufs, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
-                case 6: ok = adjoint_unit<6>(d, ul, bars, bufs, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
-                case 7: ok = adjoint_unit<7>(d, ul, bars, bufs, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
-                default: ok = adjoint_unit<8>(d, ul, bars, bufs, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
+                case 1: ok = adjoint_unit<1>(d, ul, bars, spare, ring, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
+                case 2: ok = adjoint_unit<2>(d, ul, bars, spare, ring, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
+                case 3: ok = adjoint_unit<3>(d, ul, bars, spare, ring, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
+                case 4: ok = adjoint_unit<4>(d, ul, bars, spare, ring, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
+                case 5: ok = adjoint_unit<5>(d, ul, bars, spare, ring, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
+                case 6: ok = adjoint_unit<6>(d, ul, bars, spare, ring, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
+                case 7: ok = adjoint_unit<7>(d, ul, bars, spare, ring, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
+                default: ok = adjoint_unit<8>(d, ul, bars, spare, ring, b.buf_bytes, lane, q, part, ws_floats, &g_err); break;
             }
         }
         if (!ok) break;  // a lost bulk copy: the error word says so; stop this warp

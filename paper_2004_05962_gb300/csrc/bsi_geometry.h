@@ -46,6 +46,7 @@ struct InstDesc {
     int tma_rows;        // adjoint tensor-copy path: rows per block (tma_block_rows), else 0
     int jrows;           // adjoint: tile-rows per unit (1, or 2 on the tensor-copy path)
     int ncyu;            // adjoint: unit rows, ceil(ncy / jrows)
+    int row_block;       // adjoint row-copy path: rows per block (row_block_rows)
     long long units;        // units of this instance
     long long unit_begin;   // first global unit index of this instance in its launch
     long long point_begin;  // adjoint reduce: first global grid point of this instance
@@ -58,7 +59,6 @@ struct InstDesc {
     const float* image;     // floating image [fZ][fY][fX]
     const float* gwarp;     // gradient mode: dL/dwarped [Z][Y][X]
     int fX, fY, fZ;
-    int rpad;
 };
 
 template <int MAXB>
@@ -211,12 +211,24 @@ BSI_HD int stage_buf_bytes(int dxmax) {
 }
 
 constexpr int kStoreStages = 3;   // forward: ring of staging buffers per warp (bulk stores in flight)
-constexpr int kLoadStages = 4;    // adjoint: ring of staging buffers per warp (bulk loads in flight)
+constexpr int kLoadStages = 2;    // adjoint row-copy path: ring of blocks per warp
 
-// Shared memory of one warp: forward -- the store ring; adjoint -- one 16-byte
-// mbarrier slot per stage, then the load ring.
+// Shared memory of one warp: forward -- the store ring; adjoint row-copy path --
+// a head (the stages' mbarriers, then 128 bytes of zeros), then the load ring.
+// A ring stage holds a block of rows of the instance's own x-spacing; with 9.25
+// KB stages twelve warps (three 4-warp CTAs) share an SM's shared memory.  The
+// generic kernel's rows may be longer than that: one row per block there.
+constexpr int kRowSpareOff = 64;
+constexpr int kRowHeadBytes = 256;
+constexpr int kRowStageBytes = 9472;
 BSI_HD int fwd_warp_smem(int buf_bytes) { return kStoreStages * buf_bytes; }
-BSI_HD int adj_warp_smem(int buf_bytes) { return kLoadStages * (16 + buf_bytes); }
+BSI_HD int adj_warp_smem(int stage_bytes) { return kRowHeadBytes + kLoadStages * stage_bytes; }
+BSI_HD int row_stage_bytes(int dxmax) { return imax(kRowStageBytes, stage_buf_bytes(dxmax)); }
+// Rows per block at spacing (dx, dy): as many as fit a stage, in even blocks.
+BSI_HD int row_block_rows(int dx, int dy) {
+    const int rb = imax(1, imin(imin(dy, kLanes), kRowStageBytes / stage_buf_bytes(dx)));
+    return (int)cdiv(dy, cdiv(dy, rb));
+}
 
 // Forward on the tensor-store path (one volume, three channels): when every row
 // of the field is a multiple of 16 bytes and every strip starts on a 16-byte

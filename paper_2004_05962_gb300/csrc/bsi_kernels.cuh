@@ -19,9 +19,9 @@
 // 16-byte-aligned bulk transfers.
 //
 // Adjoint (transpose of Eq. 1): the same strip walked in the opposite
-// direction.  Rows of the voxel gradient arrive by bulk copy into a ring of
-// kLoadStages buffers per warp (mbarrier completion, issued kLoadStages rows
-// ahead); each lane applies the x-transpose to its tile, a column collects
+// direction.  Blocks of rows of the voxel gradient arrive by bulk copy into a
+// ring of kLoadStages stages per warp (mbarrier completion, issued kLoadStages
+// blocks ahead); each lane applies the x-transpose to its tile, a column collects
 // the four tiles that touch it with shuffles, and y and z are accumulated in
 // registers into per-unit partial sums that a second kernel reduces in a
 // fixed order (no atomics, bitwise reproducible).
@@ -544,35 +544,41 @@ __device__ __forceinline__ void fma3(float (&q)[3], float w, float g0, float g1,
     q[2] = fmaf(w, g2, q[2]);
 }
 
-// q += w (g0, g1, g2) with three scalar FMAs.
-__device__ __forceinline__ void fma3_scalar(float (&q)[3], float w, float g0, float g1, float g2) {
-    q[0] = fmaf(w, g0, q[0]);
-    q[1] = fmaf(w, g1, q[1]);
-    q[2] = fmaf(w, g2, q[2]);
-}
+// The x-transpose's FMAs of one voxel, q_l += w_l g per channel: taps 0 and 1, 2
+// and 3 packed (their weights lie side by side in the table; the doubled operand
+// is the voxel's value), bitwise the scalar FMAs.
+// Pairs of taps measured fastest on both adjoint paths: the 64-volume batch's
+// row-copy kernel 0.448 scalar, 0.432 channels, 0.411 ms pairs; the tensor-copy
+// kernel inside a 512 x 512 x 300 step at spacing 5 0.165 -> 0.157 ms (step 0.3203
+// -> 0.3127; channels slowed that step), 512^3 at 3, 4 and 8 equal.
 
-template <bool PK>
-__device__ __forceinline__ void fma3_sel(float (&q)[3], float w, float g0, float g1, float g2) {
-    if constexpr (PK) fma3(q, w, g0, g1, g2);
-    else fma3_scalar(q, w, g0, g1, g2);
+__device__ __forceinline__ void fma_taps(float (&q4)[4][3], int wo, float g0, float g1, float g2) {
+    const float g[3] = {g0, g1, g2};
+#pragma unroll
+    for (int l = 0; l < 4; l += 2)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float2 a = __ffma2_rn(make_float2(c_lut.w[wo + l], c_lut.w[wo + l + 1]), make_float2(g[c], g[c]),
+                                        make_float2(q4[l][c], q4[l + 1][c]));
+            q4[l][c] = a.x;
+            q4[l + 1][c] = a.y;
+        }
 }
 
 // x-transpose of one voxel: q_l += B_l(r/dx) g, per channel; the voxel's three
 // channels sit at shared address sv.
-template <bool PK = true>
 __device__ __forceinline__ void gather_voxel(float (&q4)[4][3], uint32_t sv, int wo) {
     const float g0 = lds_f32(sv), g1 = lds_f32(sv + 4), g2 = lds_f32(sv + 8);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) fma3_sel<PK>(q4[l], c_lut.w[wo + l], g0, g1, g2);
+    fma_taps(q4, wo, g0, g1, g2);
 }
 
 // x-transpose of a whole tile of DX voxels read from shared address sv with
 // VW-float loads (sv aligned to 4 VW bytes; see tile_vec).
-template <int DX, int VW, bool PK = true>
+template <int DX, int VW>
 __device__ __forceinline__ void gather_tile(float (&q4)[4][3], uint32_t sv) {
     if (VW == 1) {
 #pragma unroll
-        for (int r = 0; r < DX; ++r) gather_voxel<PK>(q4, sv + 12u * r, weight_base(DX) + 4 * r);
+        for (int r = 0; r < DX; ++r) gather_voxel(q4, sv + 12u * r, weight_base(DX) + 4 * r);
     } else {
         float g[3 * DX];
 #pragma unroll
@@ -581,10 +587,7 @@ __device__ __forceinline__ void gather_tile(float (&q4)[4][3], uint32_t sv) {
             else lds_v2_f32(sv + 8 * i, g[2 * i], g[2 * i + 1]);
         }
 #pragma unroll
-        for (int r = 0; r < DX; ++r)
-#pragma unroll
-            for (int l = 0; l < 4; ++l)
-                fma3_sel<PK>(q4[l], c_lut.w[weight_base(DX) + 4 * r + l], g[3 * r], g[3 * r + 1], g[3 * r + 2]);
+        for (int r = 0; r < DX; ++r) fma_taps(q4, weight_base(DX) + 4 * r, g[3 * r], g[3 * r + 1], g[3 * r + 2]);
     }
 }
 
@@ -626,63 +629,94 @@ __device__ __forceinline__ void accumulate_z(float (&hz)[4][NR][3], const float 
     }
 }
 
+// x-transpose of a tile of DX voxels (DX a multiple of 4) whose row starts PH
+// floats past a 16-byte boundary, from the boundary at sv: whole 16-byte vectors,
+// the tile's values taken from them by position.  The lanes' tiles are 12 DX
+// bytes apart (DX = 4: no bank conflict, 8: two ways; one value per load would
+// meet four and eight).
+template <int DX, int PH>
+__device__ __forceinline__ void gather_tile_phase(float (&q4)[4][3], uint32_t sv) {
+    constexpr int NV = (3 * DX + PH + 3) / 4;
+    float g[4 * NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) lds_v4_f32(sv + 16 * i, g[4 * i], g[4 * i + 1], g[4 * i + 2], g[4 * i + 3]);
+#pragma unroll
+    for (int r = 0; r < DX; ++r)
+        fma_taps(q4, weight_base(DX) + 4 * r, g[3 * r + PH], g[3 * r + 1 + PH], g[3 * r + 2 + PH]);
+}
+
+// One adjoint unit on the row-copy path (any row alignment).  Blocks of rb rows
+// of a voxel plane (rb slots of the ring stage, one row each) arrive by one bulk
+// copy per row, lane r issuing row r's, so that the copies' address arithmetic,
+// the barrier and the wait are paid per block, not per row (with those per row,
+// and one value per load where tiles lie 48 or 96 bytes apart: 64-volume batch
+// 0.523 ms, now 0.411; 255 x 256 x 256 at spacing 8 0.165 -> 0.110, at 4 0.081 ->
+// 0.059, at 5 0.057 -> 0.050 ms).  Two stages of 9.25 KB; three of 6.2 KB made the
+// batch 0.50 ms.  Empty tiles read the warp's spare
+// zeros; a tile cut by the volume's end reads zeros written after its row.
 template <int DX>
-__device__ __forceinline__ bool adjoint_unit(const InstDesc& d, long long ul, uint64_t* bars,
-                                             unsigned char* bufs, int buf_bytes, int lane, unsigned& q,
+__device__ __forceinline__ bool adjoint_unit(const InstDesc& d, long long ul, uint64_t* bars, uint32_t spare,
+                                             unsigned char* ring, int stage_bytes, int lane, unsigned& q,
                                              float* part, long long ws_floats, unsigned* err) {
     const int dx = DX > 0 ? DX : d.dx;
     const AdjUnit u = adj_unit(d, ul);
     const int cell = u.col0 - kHalo + lane;
     const int nv = (cell >= 0 && cell < d.ncx) ? imin(dx, d.X - cell * dx) : 0;
-    // A specialised spacing reads all DX voxels of every lane, unpredicated.  In
-    // a ragged unit (a cut or empty tile: the first and last x-groups) each
-    // staged row gets zfloats zeros right after its nvox voxels; a cut tile
-    // reads its missing voxels there and an empty tile reads all of its voxels
-    // there, so both add exact zeros.  The zeros end by voxel 32 DX of the
-    // strip, inside the ring buffer.
-    const bool ragged = DX > 0 && !__all_sync(kFull, nv == dx);
-    const int zfloats = 3 * imin(dx, kLanes * dx - u.nvox);
-    // strip-local first voxel of this lane's tile (empty tiles: the zeros)
-    const int xl = (DX > 0 && nv == 0) ? u.nvox : cell * dx - u.xs;
+    const int slot = stage_buf_bytes(dx), rb = d.row_block;
+    // A specialised spacing reads all DX voxels of every lane, unpredicated: the
+    // missing voxels of a cut tile are the zeros after the row's nvox voxels.
+    const bool cut = DX > 0 && __any_sync(kFull, nv > 0 && nv < dx);
+    const int zfloats = 3 * (dx - 1);
     const int y0 = u.jy * d.dy, yn = imin(d.dy, d.Y - y0);
+    const int nblk = (yn + rb - 1) / rb;
     const int zb = u.kz0 * d.dz;
-    const int rows = (imin(u.kz1 * d.dz, d.Z) - zb) * yn;
+    const int planes = imin(u.kz1 * d.dz, d.Z) - zb;
+    const int blocks = u.nvox > 0 ? planes * nblk : 0;   // (a unit of halo columns only may read no voxel)
     const int wxb = weight_base(dx), wyb = weight_base(d.dy), wzb = weight_base(d.dz);
     const int nbytes = u.nvox * 12;
-    const long long row_pitch = 12LL * d.X;              // bytes from row y to row y + 1
-    const long long plane_pitch = row_pitch * d.Y;       // bytes from plane z to plane z + 1
+    const uintptr_t row_pitch = (uintptr_t)12 * d.X;     // bytes from row y to row y + 1
+    const uintptr_t plane_pitch = row_pitch * d.Y;       // bytes from plane z to plane z + 1
     const uintptr_t gbase = reinterpret_cast<uintptr_t>(d.grad);
     const uintptr_t A0 = ceil16(gbase);
     const uintptr_t A1 = floor16(gbase + (uintptr_t)(12LL * d.X * d.Y * d.Z));
     const uintptr_t g_first = gbase + 4 * field_elem(d, zb, y0, u.xs);   // row 0 of the unit
     // only a unit holding the first or last row of the array has bytes outside the bulk copies
     const bool unit_edge = g_first < A0 ||
-        gbase + 4 * field_elem(d, imin(u.kz1 * d.dz, d.Z) - 1, y0 + yn - 1, u.xs) + (uintptr_t)nbytes > A1;
+        g_first + (uintptr_t)(planes - 1) * plane_pitch + (uintptr_t)(yn - 1) * row_pitch + (uintptr_t)nbytes > A1;
     const unsigned q0 = q;
+    BSI_GUARD(rb >= 1 && rb <= kLanes && rb * slot <= stage_bytes, kErrStage, err) {}
 
-    // Producer (lane 0): puts the unit's rows in flight in order, row k into ring
-    // buffer (q0 + k) % kLoadStages; ig / iy / ik track the next row to issue.
-    uintptr_t ig = g_first;
-    int iy = 0, ik = 0;
-    auto issue_next = [&]() {
+    // Producer (the whole warp): puts the unit's next block in flight, block ik into
+    // stage (q0 + ik) % kLoadStages; lane r copies row r.
+    int ik = 0, ii = 0;
+    uintptr_t gp = g_first;   // row 0 of that block's plane
+    auto issue = [&]() {
         const unsigned st = (q0 + (unsigned)ik) % kLoadStages;
-        const RowLoad L = row_load(reinterpret_cast<const unsigned char*>(ig), nbytes, A0, A1);
-        if (L.s1 > L.s0) {
-            mbar_arrive_expect_tx(&bars[st], (uint32_t)(L.s1 - L.s0));
-            bulk_load(bufs + st * buf_bytes + (L.s0 - L.lo), reinterpret_cast<const void*>(L.s0),
-                      (uint32_t)(L.s1 - L.s0), &bars[st]);
-        } else {
-            mbar_arrive(&bars[st]);
+        const int r0 = ii * rb, n = imin(rb, yn - r0);
+        uint32_t bytes = 0;
+        RowLoad L = {};
+        if (lane < n) {
+            L = row_load(reinterpret_cast<const unsigned char*>(gp + (uintptr_t)(r0 + lane) * row_pitch), nbytes, A0, A1);
+            if (L.s1 > L.s0) bytes = (uint32_t)(L.s1 - L.s0);
+        }
+        const uint32_t total = __reduce_add_sync(kFull, bytes);
+        if (lane == 0) {
+            if (total > 0) mbar_arrive_expect_tx(&bars[st], total);
+            else mbar_arrive(&bars[st]);
+        }
+        __syncwarp();
+        BSI_GUARD((L.s0 - L.lo) + bytes <= (uintptr_t)slot, kErrStage, err) {
+            if (bytes > 0)
+                bulk_load(ring + st * stage_bytes + lane * slot + (L.s0 - L.lo), reinterpret_cast<const void*>(L.s0),
+                          bytes, &bars[st]);
         }
         ++ik;
-        ig += row_pitch;
-        if (++iy == yn) {
-            iy = 0;
-            ig += plane_pitch - yn * row_pitch;
+        if (++ii == nblk) {
+            ii = 0;
+            gp += plane_pitch;
         }
     };
-    if (lane == 0)
-        for (int k = 0; k < rows && k < kLoadStages; ++k) issue_next();
+    while (ik < blocks && ik < kLoadStages) issue();
     uintptr_t gz = g_first;   // consumer: first row of the current voxel plane
 
     float hz[4][4][3];
@@ -692,86 +726,89 @@ __device__ __forceinline__ bool adjoint_unit(const InstDesc& d, long long ul, ui
         for (int m = 0; m < 4; ++m)
 #pragma unroll
             for (int c = 0; c < 3; ++c) hz[n][m][c] = 0.f;
+    const uint32_t xoff = 12u * (uint32_t)(cell * dx - u.xs);   // this lane's tile in a row
+    const uint32_t stride = nv > 0 ? (uint32_t)slot : 0u;
 
     int k = 0;
     for (int kz = u.kz0; kz < u.kz1; ++kz) {
         const int z0 = kz * d.dz, zn = imin(d.dz, d.Z - z0);
-        for (int rz = 0; rz < zn; ++rz, gz += plane_pitch) {
+        for (int rz = 0; rz < (blocks > 0 ? zn : 0); ++rz, gz += plane_pitch) {
             float hy[4][3];
 #pragma unroll
             for (int m = 0; m < 4; ++m)
 #pragma unroll
                 for (int c = 0; c < 3; ++c) hy[m][c] = 0.f;
 
-            uintptr_t g = gz;
-            for (int ry = 0; ry < yn; ++ry, ++k, g += row_pitch) {
+            for (int i = 0; i < nblk; ++i, ++k) {
                 const unsigned qq = q0 + (unsigned)k;
                 const unsigned st = qq % kLoadStages;
                 if (!mbar_wait_bounded(&bars[st], (qq / kLoadStages) & 1u)) {
                     // a bulk copy never completed: record it, give the copies still
                     // in flight a bounded chance to land, and stop this warp
                     if (lane == 0) atomicOr(err, kErrTimeout);
-                    for (int p = k + 1; p < rows && p < k + kLoadStages; ++p) {
+                    for (int p = k + 1; p < ik; ++p) {
                         const unsigned qp = q0 + (unsigned)p;
                         (void)mbar_wait_bounded(&bars[qp % kLoadStages], (qp / kLoadStages) & 1u);
                     }
-                    q = q0 + (unsigned)rows;
+                    q = q0 + (unsigned)blocks;
                     return false;
                 }
-                unsigned char* sb = bufs + st * buf_bytes + (g & 15);
-                BSI_GUARD((int)(g & 15) + nbytes <= buf_bytes && g >= gbase &&
-                              (long long)(g - gbase) / 4 + 3LL * u.nvox <= 3LL * d.X * d.Y * d.Z,
-                          kErrGradRead, err) {
-                    if (unit_edge && (g < A0 || g + (uintptr_t)nbytes > A1)) {
-                        // first or last row of the array: elements outside the bulk copy
-                        const RowLoad L = row_load(reinterpret_cast<const unsigned char*>(g), nbytes, A0, A1);
-                        for (int i = lane; i < u.nvox * 3; i += kLanes) {
-                            const uintptr_t a = g + 4u * (uintptr_t)i;
-                            if (a < L.s0 || a >= L.s1)
-                                reinterpret_cast<float*>(sb)[i] = *reinterpret_cast<const float*>(a);
+                const int r0 = i * rb, rows = imin(rb, yn - r0);
+                unsigned char* blk = ring + st * stage_bytes;
+                const uintptr_t g = gz + (uintptr_t)r0 * row_pitch;
+                if (unit_edge) {   // first or last row of the array: elements outside the bulk copy
+                    for (int r = 0; r < rows; ++r) {
+                        const uintptr_t gr = g + (uintptr_t)r * row_pitch;
+                        if (gr >= A0 && gr + (uintptr_t)nbytes <= A1) continue;
+                        const RowLoad L = row_load(reinterpret_cast<const unsigned char*>(gr), nbytes, A0, A1);
+                        float* sb = reinterpret_cast<float*>(blk + r * slot + (gr & 15));
+                        for (int e = lane; e < u.nvox * 3; e += kLanes) {
+                            const uintptr_t a = gr + 4u * (uintptr_t)e;
+                            if (a < L.s0 || a >= L.s1) sb[e] = *reinterpret_cast<const float*>(a);
                         }
                     }
+                    __syncwarp();
                 }
-                BSI_GUARD((int)(g & 15) + 12 * u.nvox + 4 * zfloats <= buf_bytes, kErrStage, err) {
-                    if (ragged && lane < zfloats) sts_f32(smem_u32(sb) + 12u * (uint32_t)u.nvox + 4u * lane, 0.f);
+                uint32_t ph = (uint32_t)g & 15u;   // the row's phase
+                if (cut) {
+                    const uint32_t zb0 = smem_u32(blk) + (uint32_t)nbytes + 4u * lane;
+                    BSI_GUARD(15 + nbytes + 4 * zfloats <= slot, kErrStage, err) {
+                        for (int r = 0; r < rows; ++r)
+                            if (lane < zfloats) sts_f32(zb0 + (uint32_t)(r * slot) + ((ph + (uint32_t)r * (uint32_t)row_pitch) & 15u), 0.f);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
-                // shared address of this lane's first voxel
-                const uint32_t sv = smem_u32(sb) + 12u * (uint32_t)xl;
-                float q4[4][3];
+                uint32_t sv = nv > 0 ? smem_u32(blk) + xoff : spare;   // this lane's tile in row 0, phase apart
+                for (int r = 0; r < rows; ++r) {
+                    const int ry = r0 + r;
+                    float q4[4][3];
 #pragma unroll
-                for (int l = 0; l < 4; ++l)
+                    for (int l = 0; l < 4; ++l)
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) q4[l][c] = 0.f;
-                if (DX > 0) {  // one path for all lanes: full, cut and empty tiles
-                    constexpr int DXS = DX > 0 ? DX : 1;
-                    // 16-byte loads for DX = 4, 8 (8-byte loads for DX = 2, 6 measured slower
-                    // than scalar ones)
-                    constexpr int VW = DXS % 4 == 0 ? 4 : 1;
-                    // vector loads when every lane's start is aligned (warp-uniform): the
-                    // row start, and in a ragged unit the zeros after nvox voxels
-                    const uint32_t amask = 4 * VW - 1;
-                    if (VW > 1 && ((uint32_t)g & amask) == 0 && (!ragged || ((12u * u.nvox) & amask) == 0))
-                        gather_tile<DXS, VW>(q4, sv);
-                    else
-                        gather_tile<DXS, 1>(q4, sv);
-                } else {
-                    for (int r = 0; r < nv; ++r) gather_voxel(q4, sv + 12u * r, wxb + 4 * r);
+                        for (int c = 0; c < 3; ++c) q4[l][c] = 0.f;
+                    if constexpr (DX > 0 && DX % 4 == 0) {
+                        switch (ph >> 2) {   // warp-uniform
+                            case 0: gather_tile_phase<DX, 0>(q4, sv); break;
+                            case 1: gather_tile_phase<DX, 1>(q4, sv); break;
+                            case 2: gather_tile_phase<DX, 2>(q4, sv); break;
+                            default: gather_tile_phase<DX, 3>(q4, sv); break;
+                        }
+                    } else if constexpr (DX > 0) {
+                        gather_tile<DX, 1>(q4, sv + ph);
+                    } else {
+                        for (int v = 0; v < nv; ++v) gather_voxel(q4, sv + ph + 12u * v, wxb + 4 * v);
+                    }
+                    sv += stride;
+                    ph = (ph + (uint32_t)row_pitch) & 15u;
+                    // column sum: the column of lane l collects q4[k] of the tile k lanes below
+                    const float b0 = c_lut.w[wyb + 4 * ry], b1 = c_lut.w[wyb + 4 * ry + 1];
+                    const float b2 = c_lut.w[wyb + 4 * ry + 2], b3 = c_lut.w[wyb + 4 * ry + 3];
+                    column_sum_y(q4, hy, b0, b1, b2, b3);
                 }
-                // this ring buffer may be refilled once every lane has read it
+                // the stage may be refilled once every lane has read it
                 fence_proxy_async_smem();
                 __syncwarp();
-                // refill in pairs: after every second row the two freed ring buffers
-                // get the next two rows, one lane-0 block for both copies
-                if (lane == 0 && (k & 1) && ik < rows) {
-                    issue_next();
-                    if (ik < rows) issue_next();
-                }
-
-                // column sum: the column of lane l collects q4[k] of the tile k lanes below
-                const float b0 = c_lut.w[wyb + 4 * ry], b1 = c_lut.w[wyb + 4 * ry + 1];
-                const float b2 = c_lut.w[wyb + 4 * ry + 2], b3 = c_lut.w[wyb + 4 * ry + 3];
-                column_sum_y(q4, hy, b0, b1, b2, b3);
+                if (ik < blocks) issue();
             }
             const float a0 = c_lut.w[wzb + 4 * rz], a1 = c_lut.w[wzb + 4 * rz + 1];
             const float a2 = c_lut.w[wzb + 4 * rz + 2], a3 = c_lut.w[wzb + 4 * rz + 3];
@@ -793,7 +830,7 @@ __device__ __forceinline__ bool adjoint_unit(const InstDesc& d, long long ul, ui
     const int nk = u.kz1 - u.kz0;
 #pragma unroll
     for (int n = 0; n < 3; ++n) flush_plane(d, ul, nk + n, u, lane, hz[n], part, ws_floats, err);
-    q = q0 + (unsigned)rows;
+    q = q0 + (unsigned)blocks;
     return true;
 }
 
@@ -805,12 +842,6 @@ __device__ __forceinline__ bool adjoint_unit(const InstDesc& d, long long ul, ui
 // ahead by lane 0; a warp waits once per block.  Halo, cut and empty tiles read
 // the zeros the copy fills in outside the array, so every lane runs the same
 // unpredicated code.  Rows are summed in the same order as adjoint_unit.
-// The tensor-copy adjoint's x-transpose stays scalar (its y and z stages are
-// packed): packed, that kernel alone ran 2% faster on a 512 x 512 x 300 volume
-// at spacing 5, but a forward + adjoint step 0.8% slower (0.3254 -> 0.3280 ms,
-// three interleaved runs), where the adjoint is bound by its reads.
-constexpr bool kTmaGatherPacked = false;
-
 template <int DX, int JR>
 __device__ __forceinline__ bool adjoint_unit_tma(const InstDesc& d, const void* tmap, long long ul,
                                                  uint64_t* bars, unsigned char* ring, int stage_bytes, int stages,
@@ -899,7 +930,7 @@ __device__ __forceinline__ bool adjoint_unit_tma(const InstDesc& d, const void* 
 #pragma unroll
                         for (int c = 0; c < 3; ++c) q4[l][c] = 0.f;
                     // 16-byte loads for DX = 4, 8: shift is then 0, box rows are 16-byte multiples
-                    gather_tile<DX, DX % 4 == 0 ? 4 : 1, kTmaGatherPacked>(q4, sv + (uint32_t)(r * row_bytes));
+                    gather_tile<DX, DX % 4 == 0 ? 4 : 1>(q4, sv + (uint32_t)(r * row_bytes));
                     // the row's tile-row within the unit (0 or 1) and its offset in that tile-row
                     const int t = (JR > 1 && ry >= d.dy) ? 1 : 0;
                     const int rr = ry - t * d.dy;
