@@ -146,6 +146,7 @@ static void fill_desc(InstDesc& d, const bsi_geom& g, bool adjoint, bool bf16 = 
     if (!adjoint) {
         d.gcells = cfg.fwd_strip_tiles > 0 ? cfg.fwd_strip_tiles : fwd_strip_tiles(d.X, d.dx, bf16);
         d.nxg = empty ? 0 : (int)cdiv(d.ncx, d.gcells);
+        d.zparts = 1;
         d.units = (long long)d.ncz * d.ncy * d.nxg;
     } else {
         d.zchunk = zchunk;
@@ -188,8 +189,8 @@ static long long adj_floats(const InstDesc& d) {
     return (f + 3) & ~3LL;  // keep every instance's partials 16-byte aligned
 }
 
-// A volume of integer x-spacing above kMaxSpecializedDx as cells of any width
-// (den = 1, off = 0; bsi_cells.cuh).
+// A volume of integer spacing as cells of any width (den = 1, off = 0;
+// bsi_cells.cuh).
 static RatDesc wide_desc(const bsi_geom& g) {
     RatDesc d;
     std::memset(&d, 0, sizeof d);
@@ -215,6 +216,37 @@ static bool takes_wide(const bsi_geom& g, int n) {
     return n == 1 && g.dx > kMaxSpecializedDx && g.dy * g.dz >= kWideMinRows && !empty_volume(g);
 }
 
+// Whether the adjoint of one volume takes the kernels on cells of any width though
+// its x-spacing has a kernel of its own: small volumes, whose few units -- at least
+// three tile-planes each -- leave most warps idle and take the time of one unit's
+// rows, where a cell plan takes units as small as a plane.  Measured (us, units of
+// tile-planes -> cells): 64^3 at spacing 5 41.1 -> 11.1, at 8 66.6 -> 15.1, 128^3 at 5
+// 41.5 -> 18.2, 160 x 192 x 192 at 5 42.7 -> 28.5, 256^3 at 8 76.7 -> 62.8, 222 x 301
+// x 100 at (5, 5, 5) 34.6 -> 28.7.  Not where the units fill two thirds of the warps
+// (256^3 at 5: 88%, 46.3 against 51.5; 317 x 203 x 155 at 5: 74%, equal) or are short
+// (192 x 192 x 160 at 3, 27 rows: 26.3 against 36.9), unless most warps idle (64^3 at
+// 3: 14.1 -> 11.8).  A rule of the geometry only (a 152-SM GPU, 16-byte-aligned
+// gradient), so that a workspace query knows the answer; a tile-config entry that
+// fixes the tile-planes per unit keeps them.
+constexpr double kSmallFill = 0.65, kSmallAnyFill = 0.3;
+constexpr int kSmallRows = 48;
+static bool takes_small(const bsi_geom& g, int n) {
+    if (n != 1 || empty_volume(g) || g.dx > kMaxSpecializedDx || lookup_config(g.dx, g.dy, g.dz).adj_zchunk > 0) return false;
+    InstDesc d;
+    fill_desc(d, g, true);
+    const bool tma = d.X % 4 == 0;
+    if (tma && two_row_units(d, 1)) set_jrows(d, kTmaJrows);
+    set_zchunk(d, kMinZChunk);
+    int wps = 3 * kAdjWarpsMax;
+    if (tma) {
+        const int blk = tma_block_bytes(d.dx, d.tma_rows);
+        wps = tma_warps_per_cta(blk, tma_default_stages(blk), 0, d.jrows);
+    }
+    const double fill = (double)d.units / (152.0 * wps);
+    const int rows = kMinZChunk * d.dz * d.jrows * d.dy;
+    return fill < kSmallAnyFill || (fill < kSmallFill && rows >= kSmallRows);
+}
+
 // Workspace floats an adjoint instance may need: the most (least, with
 // `least`) over every plan the launch may pick -- tile-rows per unit 1, or also
 // kTmaJrows where the volume could take the tensor-copy path, times the table's
@@ -235,7 +267,7 @@ static long long adj_floats_bound(const bsi_geom& g, bool least = false) {
             if (fixed) break;
         }
     }
-    if (!least && takes_wide(g, 1))
+    if (!least && (takes_wide(g, 1) || takes_small(g, 1)))
         m = std::max(m, std::max(cell_plan(wide_desc(g), true, false).part_floats, cell_plan(wide_desc(g), true, true).part_floats));
     return m;
 }
@@ -474,6 +506,15 @@ static int forward_tma_rows(const InstDesc& d, bool bf16, bool generic, int c = 
     return fwd_tma_rows(d.X, d.dx, d.dy, d.gcells, bf16, c);
 }
 
+// Splits the tile-planes of a small volume's forward units (fwd_zparts), a warp
+// taking warp_smem bytes of shared memory, two CTAs on an SM at most.
+static void split_tile_planes(InstDesc& d, int warp_smem) {
+    const int wpc = warps_per_cta(warp_smem, d.warps_req);
+    const int ctas = imax(1, imin(2, kTmaSmemBudget / (wpc * warp_smem + 1024)));
+    d.zparts = fwd_zparts(d.units, (long long)device_sms() * ctas * wpc, d.dz);
+    d.units *= d.zparts;
+}
+
 enum class Op { Forward, AdjointPartials, AdjointReduce };
 
 template <int MAXB>
@@ -493,13 +534,15 @@ static cudaError_t run_group(const Group& g, Op op, bool bf16, float* part, long
         Batch<1> b;
         to_batch(g, b, op != Op::Forward);
         if (op == Op::Forward) {
-            if (bf16_odd_strips(b.inst[0], bf16, g.generic)) b.total_units = b.inst[0].units;
-            const int rb = forward_tma_rows(b.inst[0], bf16, g.generic);
-            if (rb > 0) {
-                CUtensorMap map;
-                const cudaError_t e = encode_field_map(b.inst[0], bf16, rb, &map);
-                if (e == cudaSuccess) return launch_forward_tma(b, bf16, 3, map, rb, s, nullptr);
-            }
+            InstDesc& d = b.inst[0];
+            bf16_odd_strips(d, bf16, g.generic);
+            const int rb = forward_tma_rows(d, bf16, g.generic);
+            CUtensorMap map;
+            const bool blocks = rb > 0 && encode_field_map(d, bf16, rb, &map) == cudaSuccess;
+            split_tile_planes(d, blocks ? fwd_tma_warp_smem(pad128(rb * fwd_tma_row_bytes(d.gcells, d.dx, bf16)))
+                                        : fwd_warp_smem(b.buf_bytes));
+            b.total_units = d.units;
+            if (blocks) return launch_forward_tma(b, bf16, 3, map, rb, s, nullptr);
             return launch_forward(b, bf16, g.generic, s, nullptr);
         }
         if (op == Op::AdjointPartials) {
@@ -599,7 +642,7 @@ static bsi_status adjoint_impl(const bsi_instance* inst, int n, void* ws, size_t
                                bool fixed_scratch = false) {
     bsi_status st = check_instances(inst, n, false, true, BSI_F32);
     if (st != BSI_OK) return st;
-    if (n == 1 && takes_wide(inst[0].geom, n)) {
+    if (n == 1 && (takes_wide(inst[0].geom, n) || takes_small(inst[0].geom, n))) {
         const RatDesc d = wide_desc(inst[0].geom);
         const long long have = (long long)(ws_bytes / sizeof(float));
         const CellPlan c = cell_plan(d, true, !misaligned(inst[0].grad_field, 16), fixed_scratch ? have : -1);
@@ -816,9 +859,10 @@ static void check_cells(const RatDesc& d, const CellPlan& c, bool adjoint, Range
         }
 }
 
-static void check_forward_group(const Group& g, int ob, RangeChecker& rc, bool cover) {
+static void check_forward_group(Group g, int ob, RangeChecker& rc, bool cover, bool split) {
     const int buf = stage_buf_bytes(g.dxmax);
-    for (const InstDesc& d : g.inst) {
+    for (InstDesc& d : g.inst) {
+        if (split) split_tile_planes(d, fwd_warp_smem(buf));
         const long long phi_elems = 3LL * d.nx * d.ny * d.nz;
         const long long nvox_all = (long long)d.X * d.Y * d.Z;
         std::vector<unsigned char> hit(cover ? (size_t)d.X * d.Y * d.Z : 0, 0);
@@ -835,14 +879,15 @@ static void check_forward_group(const Group& g, int ob, RangeChecker& rc, bool c
                     }
                 if (lane < u.ncell && lane * d.dx >= u.nvox) rc.fail("emitting lane past strip", lane, u.nvox);
             }
-            const int z0 = u.kz * d.dz, zn = imin(d.dz, d.Z - z0);
+            const int z0 = u.kz * d.dz, zn = imin(u.rz1, d.Z - z0);
             const int y0 = u.jy * d.dy, yn = imin(d.dy, d.Y - y0);
+            if (u.rz0 < 0 || u.rz1 > d.dz) rc.fail("planes of a part", u.rz0, u.rz1);
             // a specialised spacing stages all 32 lanes x dx voxels (past the row end too)
             const int staged = d.dx <= kMaxSpecializedDx && !g.generic ? kLanes * d.dx : u.nvox;
             if (u.nvox > staged || 15 + staged * ob > buf) rc.fail("staging overflow", staged, buf);
             if (warps_per_cta(fwd_warp_smem(buf)) * fwd_warp_smem(buf) > kSmemBudget)
                 rc.fail("forward shared memory over budget", buf, kSmemBudget);
-            for (int rz = 0; rz < zn; ++rz)
+            for (int rz = u.rz0; rz < zn; ++rz)
                 for (int ry = 0; ry < yn; ++ry) {
                     const long long v0 = field_elem(d, z0 + rz, y0 + ry, u.x0) / 3;   // voxel index
                     if (v0 < 0 || v0 + u.nvox > nvox_all) rc.fail("field write", v0, nvox_all);
@@ -962,6 +1007,29 @@ static void check_adjoint_group(const Group& g, long long ws_floats, RangeChecke
                         }
                     }
                 }
+    }
+}
+
+// The adjoint's units of tile-planes, as a call over these volumes plans them.
+static void check_adjoint_plans(const bsi_instance* inst, int n, bool cover, RangeChecker& rc) {
+    long long ws = 0;
+    const std::vector<Group> groups = plan(descs(inst, n, true, false, true), &ws, true);
+    // the documented workspace (the bound over every plan) holds the planned one
+    long long bound = 0;
+    for (int i = 0; i < n; ++i) bound += adj_floats_bound(inst[i].geom);
+    if (ws > bound) rc.fail("planned workspace over the documented bound", ws, bound);
+    // and so does the least bound the no-alloc entry point admits a volume by
+    if (n == 1) {
+        long long ws1 = 0;
+        const long long least = adj_floats_bound(inst[0].geom, true);
+        (void)plan(descs(inst, 1, true, false, true, least), &ws1, true);
+        if (ws1 > least) rc.fail("no plan fits the least bound", ws1, least);
+    }
+    for (const Group& g : groups) {
+        check_adjoint_group(g, ws, rc, cover);
+        long long total = 0;
+        for (const InstDesc& d : g.inst) total += d.units;
+        if (cover) check_slots(total, rc);
     }
 }
 
@@ -1189,14 +1257,14 @@ bsi_status bsi_scalar_forward(const bsi_geom* g, const float* coeff, void* out, 
     (void)cudaGetLastError();
     const bool bf16 = out_dtype == BSI_BF16;
     const int rb = kScalarTma && (bf16 || b.inst[0].dx != 4) ? forward_tma_rows(b.inst[0], bf16, grp.generic, 1) : 0;
-    if (rb > 0) {
-        CUtensorMap map;
-        if (encode_field_map(b.inst[0], bf16, rb, &map, 1) == cudaSuccess) {
-            const cudaError_t e = launch_forward_tma(b, bf16, 1, map, rb, reinterpret_cast<cudaStream_t>(stream), nullptr);
-            return e == cudaSuccess ? BSI_OK : cuda_fail(e);
-        }
-    }
-    const cudaError_t e = launch_forward_scalar(b, bf16, grp.generic, reinterpret_cast<cudaStream_t>(stream), nullptr);
+    CUtensorMap map;
+    const bool blocks = rb > 0 && encode_field_map(b.inst[0], bf16, rb, &map, 1) == cudaSuccess;
+    split_tile_planes(b.inst[0], blocks ? fwd_tma_warp_smem(pad128(rb * fwd_tma_row_bytes(b.inst[0].gcells, b.inst[0].dx, bf16, 1)))
+                                        : fwd_warp_smem(b.buf_bytes));
+    b.total_units = b.inst[0].units;
+    const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    const cudaError_t e = blocks ? launch_forward_tma(b, bf16, 1, map, rb, s, nullptr)
+                                 : launch_forward_scalar(b, bf16, grp.generic, s, nullptr);
     return e == cudaSuccess ? BSI_OK : cuda_fail(e);
 }
 
@@ -1386,8 +1454,8 @@ int bsi_selfcheck_ranges(const bsi_instance* inst, int n, int op, int cover, cha
         for (int i = 0; i < n; ++i) ok = ok && check_geom(&inst[i].geom) == BSI_OK;
         if (!ok) {
             rc.fail("invalid geometry", n, 0);
-        } else if ((op == 0 || op == 2) && n == 1 && takes_wide(inst[0].geom, n)) {
-            // cells of any width, for aligned and unaligned arrays, and within the least no-alloc plan
+        } else if (n == 1 && (((op == 0 || op == 2) && takes_wide(inst[0].geom, n)) || (op == 2 && takes_small(inst[0].geom, n)))) {
+            // cells of any width, for aligned and unaligned arrays
             const RatDesc d = wide_desc(inst[0].geom);
             const long long bound = adj_floats_bound(inst[0].geom);
             for (int vec = 0; vec < 2; ++vec) {
@@ -1395,6 +1463,8 @@ int bsi_selfcheck_ranges(const bsi_instance* inst, int n, int op, int cover, cha
                 check_cells(d, c, op == 2, rc, cover != 0);
                 if (c.part_floats > bound) rc.fail("planned workspace over the documented bound", c.part_floats, bound);
             }
+            // where the fixed scratch does not hold those, and in batches, units of tile-planes
+            if (op == 2 && takes_small(inst[0].geom, n)) check_adjoint_plans(inst, n, cover != 0, rc);
         } else if (op != 2) {
             std::vector<InstDesc> all = descs(inst, n, false, op == 1 || op == 6);
             all.erase(std::remove_if(all.begin(), all.end(), [](const InstDesc& d) { return d.units == 0; }),
@@ -1402,7 +1472,7 @@ int bsi_selfcheck_ranges(const bsi_instance* inst, int n, int op, int cover, cha
             for (const Group& g : plan(all, nullptr)) {
                 // staging bytes per voxel: the field (12 FP32, 6 BF16), T for both
                 // resampling modes (12), the scalar forward (4 FP32, 2 BF16)
-                check_forward_group(g, op == 1 ? 6 : op == 5 ? 4 : op == 6 ? 2 : 12, rc, cover != 0);
+                check_forward_group(g, op == 1 ? 6 : op == 5 ? 4 : op == 6 ? 2 : 12, rc, cover != 0, n == 1 && op != 3 && op != 4);
                 // the single-volume forward's tensor-store path (3 or 1 channels)
                 if ((op == 0 || op == 1 || op == 5 || op == 6) && n == 1 && g.inst.size() == 1 && !g.generic)
                     check_forward_tma(g.inst[0], op == 1 || op == 6, op >= 5 ? 1 : 3, rc);
@@ -1411,25 +1481,7 @@ int bsi_selfcheck_ranges(const bsi_instance* inst, int n, int op, int cover, cha
                 if (cover) check_slots(total, rc);
             }
         } else {
-            long long ws = 0;
-            const std::vector<Group> groups = plan(descs(inst, n, true, false, true), &ws, true);
-            // the documented workspace (the bound over every plan) holds the planned one
-            long long bound = 0;
-            for (int i = 0; i < n; ++i) bound += adj_floats_bound(inst[i].geom);
-            if (ws > bound) rc.fail("planned workspace over the documented bound", ws, bound);
-            // and so does the least bound the no-alloc entry point admits a volume by
-            if (n == 1) {
-                long long ws1 = 0;
-                const long long least = adj_floats_bound(inst[0].geom, true);
-                (void)plan(descs(inst, 1, true, false, true, least), &ws1, true);
-                if (ws1 > least) rc.fail("no plan fits the least bound", ws1, least);
-            }
-            for (const Group& g : groups) {
-                check_adjoint_group(g, ws, rc, cover != 0);
-                long long total = 0;
-                for (const InstDesc& d : g.inst) total += d.units;
-                if (cover) check_slots(total, rc);
-            }
+            check_adjoint_plans(inst, n, cover != 0, rc);
         }
     }
     if (msg && msg_len) {

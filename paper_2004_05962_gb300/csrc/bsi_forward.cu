@@ -15,7 +15,7 @@ static __device__ unsigned g_err;
 // narrow volumes fill 63% of the lanes, so the per-row instructions bound them.
 constexpr bool kBatchFwdPacked = true;
 
-template <int MAXB, bool BF16, bool GENERIC, int C = 3>
+template <int MAXB, bool BF16, bool GENERIC, int C = 3, bool PARTS = MAXB == 1>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * kLanes, 2)
     bsi_forward_kernel(const __grid_constant__ Batch<MAXB> b) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -39,17 +39,17 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * kLanes, 2)
         const InstDesc& dc = b.inst[BF16 ? ii : inst_index<MAXB>(ii)];
         const long long ul = uu - d.unit_begin;
         if (GENERIC) {
-            forward_unit<0, BF16, C, PA>(d, ul, stage, b.buf_bytes, lane, ring, &g_err);
+            forward_unit<0, BF16, C, PA, PARTS>(d, ul, stage, b.buf_bytes, lane, ring, &g_err);
         } else {
             switch (d.dx) {
-                case 1: forward_unit<1, BF16, C, PA>(dc, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
-                case 2: forward_unit<2, BF16, C, PA>(dc, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
-                case 3: forward_unit<3, BF16, C, PA>(dc, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
-                case 4: forward_unit<4, BF16, C, PA>(d, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
-                case 5: forward_unit<5, BF16, C, PA>(d, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
-                case 6: forward_unit<6, BF16, C, PA>(d, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
-                case 7: forward_unit<7, BF16, C, PA>(d, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
-                default: forward_unit<8, BF16, C, PA>(d, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
+                case 1: forward_unit<1, BF16, C, PA, PARTS>(dc, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
+                case 2: forward_unit<2, BF16, C, PA, PARTS>(dc, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
+                case 3: forward_unit<3, BF16, C, PA, PARTS>(dc, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
+                case 4: forward_unit<4, BF16, C, PA, PARTS>(d, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
+                case 5: forward_unit<5, BF16, C, PA, PARTS>(d, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
+                case 6: forward_unit<6, BF16, C, PA, PARTS>(d, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
+                case 7: forward_unit<7, BF16, C, PA, PARTS>(d, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
+                default: forward_unit<8, BF16, C, PA, PARTS>(d, ul, stage, b.buf_bytes, lane, ring, &g_err); break;
             }
         }
     }
@@ -59,9 +59,9 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * kLanes, 2)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // this CTA's rows are written
 }
 
-template <int MAXB, bool BF16, bool GENERIC, int C = 3>
+template <int MAXB, bool BF16, bool GENERIC, int C = 3, bool PARTS = MAXB == 1>
 static cudaError_t launch_fwd_t(const Batch<MAXB>& b, cudaStream_t s, LaunchInfo* info) {
-    auto kern = bsi_forward_kernel<MAXB, BF16, GENERIC, C>;
+    auto kern = bsi_forward_kernel<MAXB, BF16, GENERIC, C, PARTS>;
     const int wpc = warps_per_cta(fwd_warp_smem(b.buf_bytes), b.warps_req);
     const int threads = wpc * kLanes;
     const int smem = wpc * fwd_warp_smem(b.buf_bytes);
@@ -148,11 +148,16 @@ cudaError_t launch_forward_tma(const Batch<1>& b, bool bf16, int channels, const
     return bf16 ? launch_fwd_tma_t<true, 3>(b, map, rb, s, info) : launch_fwd_tma_t<false, 3>(b, map, rb, s, info);
 }
 
-// Scalar (one-channel) interpolation of a single volume.
+// Scalar (one-channel) interpolation of a single volume.  FP32 units of whole
+// tile-planes have a kernel of their own: finding a unit's part costs the large
+// ones, a few rows each, 1.4% (4x zoom to 512 x 512 x 300 70.1 against 71.1 us); no
+// other kernel shows it.
 cudaError_t launch_forward_scalar(const Batch<1>& b, bool bf16, bool generic, cudaStream_t s, LaunchInfo* info) {
     if (bf16)
         return generic ? launch_fwd_t<1, true, true, 1>(b, s, info) : launch_fwd_t<1, true, false, 1>(b, s, info);
-    return generic ? launch_fwd_t<1, false, true, 1>(b, s, info) : launch_fwd_t<1, false, false, 1>(b, s, info);
+    if (generic) return launch_fwd_t<1, false, true, 1>(b, s, info);
+    return b.inst[0].zparts > 1 ? launch_fwd_t<1, false, false, 1>(b, s, info)
+                                : launch_fwd_t<1, false, false, 1, false>(b, s, info);
 }
 
 template cudaError_t launch_forward<1>(const Batch<1>&, bool, bool, cudaStream_t, LaunchInfo*);

@@ -42,6 +42,7 @@ struct InstDesc {
     int nzc;             // adjoint: tile-plane chunks
     int zchunk;          // adjoint: tile-planes per chunk
     int gcells;          // forward: tiles per warp strip (<= 29; see fwd_strip_tiles)
+    int zparts;          // forward: units per tile-plane of a strip (see fwd_zparts)
     int warps_req;       // requested warps per CTA from the tile-config table (0: automatic)
     int tma_rows;        // adjoint tensor-copy path: rows per block (tma_block_rows), else 0
     int jrows;           // adjoint: tile-rows per unit (1, or 2 on the tensor-copy path)
@@ -120,6 +121,7 @@ BSI_HD long long slot_unit(long long r, int cta, int warp, int ctas, int wpc, lo
 
 struct FwdUnit {
     int kz, jy, xg;
+    int rz0, rz1;   // planes of the tile-plane the unit takes
     int cell0;   // first tile of the strip; lane l holds grid column cell0 + l
     int ncell;   // tiles the warp outputs (<= 29)
     int x0;      // first voxel of the strip
@@ -143,6 +145,21 @@ BSI_HD int fwd_strip_tiles(int X, int dx, bool bf16) {
     return kGroupCells;
 }
 
+// Units per tile-plane of a strip, one volume of `units` whole ones on `slots`
+// resident warps: a volume of fewer strips than warps is bound by the serial walk
+// of a unit's dy dz rows, not by bandwidth, and its tile-planes are split so that
+// every warp gets a part (one volume per call; us for whole tile-planes -> parts:
+// 64^3 at spacing 5 10.6 -> 4.2, at 8 34.0 -> 6.8; 128^3 at 5 10.6 -> 7.8; 160 x
+// 192 x 192 at 8 34.3 -> 14.2).  From as many units as warps on, parts only add
+// their start, 48 loads of control points: 160 x 192 x 192 at 5 22.7 us whole, 21.4
+// and 22.9 in 2 and 5 parts, 256^3 at 5 36.4, 37.7 and 45.5.
+BSI_HD int fwd_zparts(long long units, long long slots, int dz) {
+    if (units <= 0 || units >= slots) return 1;
+    const long long p = slots / units;
+    return p < dz ? (int)p : dz;
+}
+
+template <bool PARTS = true>
 BSI_HD FwdUnit fwd_unit(const InstDesc& d, long long ul) {
     FwdUnit u;
     if (d.units <= 0x7fffffffLL) {   // 32-bit division (64-bit division is a long sequence)
@@ -155,6 +172,15 @@ BSI_HD FwdUnit fwd_unit(const InstDesc& d, long long ul) {
         const long long t = ul / d.nxg;
         u.jy = (int)(t % d.ncy);
         u.kz = (int)(t / d.ncy);
+    }
+    u.rz0 = 0;
+    u.rz1 = d.dz;
+    if (PARTS && d.zparts > 1) {
+        const int zp = u.kz;
+        u.kz = zp / d.zparts;
+        const int p = zp - u.kz * d.zparts;
+        u.rz0 = d.dz * p / d.zparts;
+        u.rz1 = d.dz * (p + 1) / d.zparts;
     }
     u.cell0 = u.xg * d.gcells;
     u.ncell = imin(d.gcells, d.ncx - u.cell0);

@@ -261,15 +261,16 @@ __device__ __forceinline__ void emit_tile(uint32_t sv, const float (&p0)[C], con
 // DX == 0 reads the spacing at run time.  ring is the warp's next staging
 // buffer in its store ring (0 .. kStoreStages - 1).  C channels per control
 // point and voxel: 3 (the displacement field) or 1 (scalar interpolation,
-// layouts [nz][ny][nx] and [Z][Y][X]).
-template <int DX, bool BF16, int C = 3, bool PACK_ALL = false>
+// layouts [nz][ny][nx] and [Z][Y][X]).  PARTS: units may be parts of tile-planes
+// (fwd_zparts; one volume per call).
+template <int DX, bool BF16, int C = 3, bool PACK_ALL = false, bool PARTS = true>
 __device__ __forceinline__ void forward_unit(const InstDesc& d, long long ul, unsigned char* stage,
                                              int buf_bytes, int lane, int& ring, unsigned* err) {
     static_assert(C == 1 || C == 3, "one (scalar) or three (displacement) channels");
     constexpr int ES = BF16 ? 2 : 4;
     constexpr bool PK = PACK_ALL || fwd_packed<DX, BF16>();
     const int dx = DX > 0 ? DX : d.dx;
-    const FwdUnit u = fwd_unit(d, ul);
+    const FwdUnit u = fwd_unit<PARTS>(d, ul);
     const int col = u.cell0 + lane;
 
     // 4 (z) x 4 (y) neighbourhood column of control points, C channels.
@@ -303,7 +304,7 @@ __device__ __forceinline__ void forward_unit(const InstDesc& d, long long ul, un
             }
         }
 
-    const int z0 = u.kz * d.dz, zn = imin(d.dz, d.Z - z0);
+    const int z0 = u.kz * d.dz, zn = imin(u.rz1, d.Z - z0);
     const int y0 = u.jy * d.dy, yn = imin(d.dy, d.Y - y0);
     const int wzb = weight_base(d.dz), wyb = weight_base(d.dy), wxb = weight_base(dx);
     const int xl = lane * dx;                 // first strip voxel of this lane's tile
@@ -313,11 +314,11 @@ __device__ __forceinline__ void forward_unit(const InstDesc& d, long long ul, un
     const long long row_pitch = (long long)C * d.X * ES;   // bytes from row y to row y + 1
     const long long plane_pitch = row_pitch * d.Y;       // bytes from plane z to plane z + 1
     unsigned char* gplane =
-        static_cast<unsigned char*>(d.field) + ((((long long)z0 * d.Y + y0) * d.X + u.x0) * C) * ES;   // field_elem for C
+        static_cast<unsigned char*>(d.field) + ((((long long)(z0 + u.rz0) * d.Y + y0) * d.X + u.x0) * C) * ES;   // field_elem for C
     // every row of the unit starts on a 16-byte boundary (x0 is a multiple of DX)
     const bool direct = C == 1 && (reinterpret_cast<uintptr_t>(d.field) & 15) == 0 && (d.X & 3) == 0;
 
-    for (int rz = 0; rz < zn; ++rz, gplane += plane_pitch) {
+    for (int rz = u.rz0; rz < zn; ++rz, gplane += plane_pitch) {
         const float a0 = c_lut.w[wzb + 4 * rz], a1 = c_lut.w[wzb + 4 * rz + 1];
         const float a2 = c_lut.w[wzb + 4 * rz + 2], a3 = c_lut.w[wzb + 4 * rz + 3];
         float pz[4][C];
@@ -442,7 +443,7 @@ __device__ __forceinline__ void forward_unit_tma(const InstDesc& d, const void* 
             ph[n][m][C > 2 ? 2 : 0] = C > 2 ? c : a;
         }
 
-    const int z0 = u.kz * d.dz, zn = imin(d.dz, d.Z - z0);
+    const int z0 = u.kz * d.dz, zn = imin(u.rz1, d.Z - z0);
     const int y0 = u.jy * d.dy, yn = imin(d.dy, d.Y - y0);
     const int wzb = weight_base(d.dz), wyb = weight_base(d.dy);
     const int rowb = d.gcells * DX * C * ES;           // row pitch of a block: the strip's bytes
@@ -451,7 +452,7 @@ __device__ __forceinline__ void forward_unit_tma(const InstDesc& d, const void* 
     const uint32_t lane_off = lane < d.gcells ? (uint32_t)(lane * DX * C * ES) : (uint32_t)(kStoreStages * blk_bytes);
     BSI_GUARD(rowb * rb <= blk_bytes && (u.x0 * C * ES) % 16 == 0, kErrStage, err) {}
 
-    for (int rz = 0; rz < zn; ++rz) {
+    for (int rz = u.rz0; rz < zn; ++rz) {
         const float a0 = c_lut.w[wzb + 4 * rz], a1 = c_lut.w[wzb + 4 * rz + 1];
         const float a2 = c_lut.w[wzb + 4 * rz + 2], a3 = c_lut.w[wzb + 4 * rz + 3];
         float pz[4][C];

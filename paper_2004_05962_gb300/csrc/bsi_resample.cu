@@ -118,7 +118,7 @@ __device__ __forceinline__ void resample_unit(const InstDesc& d, long long ul, u
             ph[ph_index(n, m, 2, lane)] = c;
         }
 
-    const int z0 = u.kz * d.dz, zn = imin(d.dz, d.Z - z0);
+    const int z0 = u.kz * d.dz, zn = imin(u.rz1, d.Z - z0);
     const int y0 = u.jy * d.dy, yn = imin(d.dy, d.Y - y0);
     const int wzb = weight_base(d.dz), wyb = weight_base(d.dy), wxb = weight_base(dx);
     const int xl = lane * dx;                 // first strip voxel of this lane's tile
@@ -127,7 +127,7 @@ __device__ __forceinline__ void resample_unit(const InstDesc& d, long long ul, u
     const uint32_t sv = s0 + 12u * (uint32_t)xl;
     BSI_GUARD((DX > 0 ? 12 * kLanes * DX : 12 * u.nvox) <= buf_bytes && (s0 & 15) == 0, kErrStage, err) {}
 
-    for (int rz = 0; rz < zn; ++rz) {
+    for (int rz = u.rz0; rz < zn; ++rz) {
         const float a0 = c_lut.w[wzb + 4 * rz], a1 = c_lut.w[wzb + 4 * rz + 1];
         const float a2 = c_lut.w[wzb + 4 * rz + 2], a3 = c_lut.w[wzb + 4 * rz + 3];
         float pz[4][3];
