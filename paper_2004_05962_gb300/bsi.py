@@ -14,6 +14,7 @@ The function names are those of the C entry points.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 
 import torch
@@ -198,9 +199,33 @@ def make_geom(shape, spacing) -> BsiGeom:
     return g
 
 
+@functools.lru_cache(maxsize=1024)
+def _geometry(shape, spacing):
+    """(grid dims + (3,), geometry, its status) of integer tuples.  A registration calls
+    with the same few geometries over and over: building one takes 4 us, a tenth of a
+    small volume's step.  The struct is only ever read."""
+    g = BsiGeom()
+    (Z, Y, X), (dz, dy, dx) = shape, spacing
+    grid = grid_shape(shape, spacing) + (3,)
+    return grid, g, library().bsi_geom_init(ctypes.byref(g), X, Y, Z, dx, dy, dz)
+
+
+def _geom_ref(g, st, shape, spacing):
+    """A pointer to a geometry of _geometry, once the tensors have been checked."""
+    if st:
+        raise BsiError(st, "bsi_geom_init", f"shape={shape} spacing={spacing}")
+    return ctypes.byref(g)
+
+
+def _ints(values):
+    return tuple(map(int, values))
+
+
 def _stream(stream, device) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream(device)
+        # (the raw handle: a Stream object takes 2 us to make)
+        return torch._C._cuda_getCurrentRawStream(device.index) if device is not None and device.index is not None \
+            else torch.cuda.current_stream(device).cuda_stream
     return int(stream.cuda_stream)
 
 
@@ -215,7 +240,7 @@ def _need(t, name, dtype, shape=None):
         raise ValueError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != tuple(shape):
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
@@ -233,13 +258,14 @@ def _out_dtype_code(dtype):
 
 def bsi_field_forward(phi, shape, spacing, out=None, out_dtype=torch.float32, stream=None):
     """Dense field [Z, Y, X, 3] from the control grid ``phi`` [nz, ny, nx, 3] (Eq. 1)."""
-    shape = tuple(int(s) for s in shape)
-    _need(phi, "phi", torch.float32, grid_shape(shape, spacing) + (3,))
+    shape = _ints(shape)
+    grid, g, gst = _geometry(shape, _ints(spacing))
+    _need(phi, "phi", torch.float32, grid)
     if out is None:
         out = torch.empty(shape + (3,), dtype=out_dtype, device=phi.device)
-    _need(out, "out", out.dtype, shape + (3,))
-    g = make_geom(shape, spacing)
-    st = library().bsi_field_forward(ctypes.byref(g), phi.data_ptr(), out.data_ptr(),
+    else:
+        _need(out, "out", out.dtype, shape + (3,))
+    st = library().bsi_field_forward(_geom_ref(g, gst, shape, spacing), phi.data_ptr(), out.data_ptr(),
                                      _out_dtype_code(out.dtype), _stream(stream, phi.device))
     _check(st, "bsi_field_forward")
     return out
@@ -268,14 +294,15 @@ def bsi_field_adjoint(grad_field, spacing, out=None, workspace=None, stream=None
     if grad_field.dim() != 4 or grad_field.shape[3] != 3:
         raise ValueError("grad_field must be [Z, Y, X, 3]")
     shape = tuple(grad_field.shape[:3])
-    grid = grid_shape(shape, spacing)
+    grid, g, gst = _geometry(shape, _ints(spacing))
     if out is None:
-        out = torch.empty(grid + (3,), dtype=torch.float32, device=grad_field.device)
-    _need(out, "out", torch.float32, grid + (3,))
-    g = make_geom(shape, spacing)
-    need = int(library().bsi_adjoint_workspace_bytes(ctypes.byref(g)))
+        out = torch.empty(grid, dtype=torch.float32, device=grad_field.device)
+    else:
+        _need(out, "out", torch.float32, grid)
+    ref = _geom_ref(g, gst, shape, spacing)
+    need = int(library().bsi_adjoint_workspace_bytes(ref))
     ws, wsb = _workspace(need, grad_field.device, workspace)
-    st = library().bsi_field_adjoint(ctypes.byref(g), grad_field.data_ptr(), out.data_ptr(),
+    st = library().bsi_field_adjoint(ref, grad_field.data_ptr(), out.data_ptr(),
                                      ws.data_ptr() if ws is not None else None, wsb,
                                      _stream(stream, grad_field.device))
     _check(st, "bsi_field_adjoint")
@@ -290,12 +317,13 @@ def bsi_field_adjoint_noalloc(grad_field, spacing, out=None, stream=None):
     if grad_field.dim() != 4 or grad_field.shape[3] != 3:
         raise ValueError("grad_field must be [Z, Y, X, 3]")
     shape = tuple(grad_field.shape[:3])
-    grid = grid_shape(shape, spacing)
+    grid, g, gst = _geometry(shape, _ints(spacing))
     if out is None:
-        out = torch.empty(grid + (3,), dtype=torch.float32, device=grad_field.device)
-    _need(out, "out", torch.float32, grid + (3,))
-    g = make_geom(shape, spacing)
-    st = library().bsi_field_adjoint_noalloc(ctypes.byref(g), grad_field.data_ptr(), out.data_ptr(),
+        out = torch.empty(grid, dtype=torch.float32, device=grad_field.device)
+    else:
+        _need(out, "out", torch.float32, grid)
+    ref = _geom_ref(g, gst, shape, spacing)
+    st = library().bsi_field_adjoint_noalloc(ref, grad_field.data_ptr(), out.data_ptr(),
                                              _stream(stream, grad_field.device))
     _check(st, "bsi_field_adjoint_noalloc")
     return out
@@ -305,20 +333,27 @@ def _instances(shapes, spacings, phis=None, fields=None, grads=None, dphis=None)
     n = len(shapes)
     arr = (BsiInstance * max(n, 1))()
     for i in range(n):
-        arr[i].geom = make_geom(shapes[i], spacings[i])
-        arr[i].phi = phis[i].data_ptr() if phis is not None else None
-        arr[i].field = fields[i].data_ptr() if fields is not None else None
-        arr[i].grad_field = grads[i].data_ptr() if grads is not None else None
-        arr[i].grad_phi = dphis[i].data_ptr() if dphis is not None else None
+        _, g, gst = _geometry(_ints(shapes[i]), _ints(spacings[i]))
+        _geom_ref(g, gst, shapes[i], spacings[i])
+        a = arr[i]
+        a.geom = g   # (copied)
+        if phis is not None:
+            a.phi = phis[i].data_ptr()
+        if fields is not None:
+            a.field = fields[i].data_ptr()
+        if grads is not None:
+            a.grad_field = grads[i].data_ptr()
+        if dphis is not None:
+            a.grad_phi = dphis[i].data_ptr()
     return arr
 
 
 def bsi_field_forward_batched(phis, shapes, spacings, outs=None, out_dtype=torch.float32, stream=None):
     """Forward over a batch of volumes of uneven size and spacing (persistent launch)."""
     n = len(phis)
-    shapes = [tuple(int(s) for s in sh) for sh in shapes]
+    shapes = [_ints(sh) for sh in shapes]
     for i in range(n):
-        _need(phis[i], f"phis[{i}]", torch.float32, grid_shape(shapes[i], spacings[i]) + (3,))
+        _need(phis[i], f"phis[{i}]", torch.float32, _geometry(shapes[i], _ints(spacings[i]))[0])
     if outs is None:
         outs = [torch.empty(shapes[i] + (3,), dtype=out_dtype, device=phis[i].device) for i in range(n)]
     dt = outs[0].dtype if n else out_dtype
@@ -344,10 +379,10 @@ def bsi_field_adjoint_batched(grads, spacings, outs=None, workspace=None, stream
         _need(grads[i], f"grads[{i}]", torch.float32)
         shapes.append(tuple(grads[i].shape[:3]))
     if outs is None:
-        outs = [torch.empty(grid_shape(shapes[i], spacings[i]) + (3,), dtype=torch.float32,
+        outs = [torch.empty(_geometry(shapes[i], _ints(spacings[i]))[0], dtype=torch.float32,
                             device=grads[i].device) for i in range(n)]
     for i in range(n):
-        _need(outs[i], f"outs[{i}]", torch.float32, grid_shape(shapes[i], spacings[i]) + (3,))
+        _need(outs[i], f"outs[{i}]", torch.float32, _geometry(shapes[i], _ints(spacings[i]))[0])
     arr = _instances(shapes, spacings, grads=grads, dphis=outs)
     dev = grads[0].device if n else torch.device("cuda")
     need = int(library().bsi_batched_adjoint_workspace_bytes(arr, n))
@@ -368,6 +403,16 @@ def make_geom_rational(shape, num, den, off):
     return g
 
 
+@functools.lru_cache(maxsize=1024)
+def _geometry_rational(shape, num, den, off):
+    """(grid dims + (3,), geometry, its status) of integer tuples (see _geometry)."""
+    arr = lambda a: (ctypes.c_int32 * 3)(*a[::-1])   # to (x, y, z)
+    g = BsiGeomRational()
+    grid = rational_grid_shape(shape, num, den, off) + (3,)
+    Z, Y, X = shape
+    return grid, g, library().bsi_geom_rational_init(ctypes.byref(g), X, Y, Z, arr(num), arr(den), arr(off))
+
+
 def rational_grid_shape(shape, num, den, off):
     """Stored grid (nz, ny, nx) for spacing num/den and lattice shift off/den voxels
     per axis ((z, y, x) order): floor(((N - 1) den + off) / num) + 4."""
@@ -378,12 +423,14 @@ def rational_grid_shape(shape, num, den, off):
 def bsi_field_forward_rational(phi, shape, num, den, off=(0, 0, 0), out=None, stream=None):
     """Eq. 1 with non-integer spacing num/den and lattice shift off/den voxels per
     axis ((z, y, x) order like ``shape``): FP32 field [Z, Y, X, 3]."""
-    shape = tuple(int(s) for s in shape)
-    _need(phi, "phi", torch.float32, rational_grid_shape(shape, num, den, off) + (3,))
+    shape = _ints(shape)
+    grid, g, gst = _geometry_rational(shape, _ints(num), _ints(den), _ints(off))
+    _need(phi, "phi", torch.float32, grid)
     if out is None:
         out = torch.empty(shape + (3,), dtype=torch.float32, device=phi.device)
-    _need(out, "out", torch.float32, shape + (3,))
-    g = make_geom_rational(shape, num, den, off)
+    else:
+        _need(out, "out", torch.float32, shape + (3,))
+    _check(gst, "bsi_geom_rational_init")
     st = library().bsi_field_forward_rational(ctypes.byref(g), phi.data_ptr(), out.data_ptr(),
                                               _stream(stream, phi.device))
     _check(st, "bsi_field_forward_rational")
@@ -400,12 +447,13 @@ def bsi_field_adjoint_rational(grad_field, num, den, off=(0, 0, 0), out=None, wo
     _need(grad_field, "grad_field", torch.float32)
     if grad_field.dim() != 4 or grad_field.shape[3] != 3:
         raise ValueError("grad_field must be [Z, Y, X, 3]")
-    shape = tuple(int(s) for s in grad_field.shape[:3])
-    grid = rational_grid_shape(shape, num, den, off)
+    shape = tuple(grad_field.shape[:3])
+    grid, g, gst = _geometry_rational(shape, _ints(num), _ints(den), _ints(off))
     if out is None:
-        out = torch.empty(grid + (3,), dtype=torch.float32, device=grad_field.device)
-    _need(out, "out", torch.float32, grid + (3,))
-    g = make_geom_rational(shape, num, den, off)
+        out = torch.empty(grid, dtype=torch.float32, device=grad_field.device)
+    else:
+        _need(out, "out", torch.float32, grid)
+    _check(gst, "bsi_geom_rational_init")
     nbytes = int(library().bsi_rational_adjoint_workspace_bytes(ctypes.byref(g)))
     ws, wsb = _workspace(nbytes, grad_field.device, workspace)
     st = library().bsi_field_adjoint_rational(ctypes.byref(g), grad_field.data_ptr(), out.data_ptr(),
@@ -437,13 +485,14 @@ def bsi_field_forward_variant(phi, shape, spacing, variant="ttli", out=None, str
 def bsi_scalar_forward(coeff, shape, spacing, out=None, out_dtype=torch.float32, stream=None):
     """Scalar BSI (image interpolation / zooming): [Z, Y, X] from a one-channel
     control grid ``coeff`` [nz, ny, nx] (Eq. 1 with one channel)."""
-    shape = tuple(int(s) for s in shape)
-    _need(coeff, "coeff", torch.float32, grid_shape(shape, spacing))
+    shape = _ints(shape)
+    grid, g, gst = _geometry(shape, _ints(spacing))
+    _need(coeff, "coeff", torch.float32, grid[:3])
     if out is None:
         out = torch.empty(shape, dtype=out_dtype, device=coeff.device)
-    _need(out, "out", out.dtype, shape)
-    g = make_geom(shape, spacing)
-    st = library().bsi_scalar_forward(ctypes.byref(g), coeff.data_ptr(), out.data_ptr(), _out_dtype_code(out.dtype),
+    else:
+        _need(out, "out", out.dtype, shape)
+    st = library().bsi_scalar_forward(_geom_ref(g, gst, shape, spacing), coeff.data_ptr(), out.data_ptr(), _out_dtype_code(out.dtype),
                                       _stream(stream, coeff.device))
     _check(st, "bsi_scalar_forward")
     return out
@@ -460,14 +509,15 @@ def _floating(image):
 def bsi_resample_forward(phi, shape, spacing, image, out=None, stream=None):
     """Floating ``image`` [fZ, fY, fX] sampled at x + T(x) (T: Eq. 1 from ``phi``),
     trilinear with zeros outside the image: warped [Z, Y, X], without storing T."""
-    shape = tuple(int(s) for s in shape)
-    _need(phi, "phi", torch.float32, grid_shape(shape, spacing) + (3,))
+    shape = _ints(shape)
+    grid, g, gst = _geometry(shape, _ints(spacing))
+    _need(phi, "phi", torch.float32, grid)
     fX, fY, fZ = _floating(image)
     if out is None:
         out = torch.empty(shape, dtype=torch.float32, device=phi.device)
-    _need(out, "out", torch.float32, shape)
-    g = make_geom(shape, spacing)
-    st = library().bsi_resample_forward(ctypes.byref(g), phi.data_ptr(), image.data_ptr(), fX, fY, fZ,
+    else:
+        _need(out, "out", torch.float32, shape)
+    st = library().bsi_resample_forward(_geom_ref(g, gst, shape, spacing), phi.data_ptr(), image.data_ptr(), fX, fY, fZ,
                                         out.data_ptr(), _stream(stream, phi.device))
     _check(st, "bsi_resample_forward")
     return out
@@ -480,17 +530,19 @@ def bsi_resample_backward_workspace_bytes(shape, spacing) -> int:
 
 def bsi_resample_backward(phi, shape, spacing, image, grad_warped, out=None, workspace=None, stream=None):
     """dL/dphi [nz, ny, nx, 3] for dL/dwarped = ``grad_warped`` [Z, Y, X]."""
-    shape = tuple(int(s) for s in shape)
-    _need(phi, "phi", torch.float32, grid_shape(shape, spacing) + (3,))
+    shape = _ints(shape)
+    grid, g, gst = _geometry(shape, _ints(spacing))
+    _need(phi, "phi", torch.float32, grid)
     _need(grad_warped, "grad_warped", torch.float32, shape)
     fX, fY, fZ = _floating(image)
     if out is None:
         out = torch.empty_like(phi)
-    _need(out, "out", torch.float32, tuple(phi.shape))
-    g = make_geom(shape, spacing)
-    need = int(library().bsi_resample_backward_workspace_bytes(ctypes.byref(g)))
+    else:
+        _need(out, "out", torch.float32, grid)
+    ref = _geom_ref(g, gst, shape, spacing)
+    need = int(library().bsi_resample_backward_workspace_bytes(ref))
     ws, wsb = _workspace(need, phi.device, workspace)
-    st = library().bsi_resample_backward(ctypes.byref(g), phi.data_ptr(), image.data_ptr(), fX, fY, fZ,
+    st = library().bsi_resample_backward(ref, phi.data_ptr(), image.data_ptr(), fX, fY, fZ,
                                          grad_warped.data_ptr(), out.data_ptr(),
                                          ws.data_ptr() if ws is not None else None, wsb,
                                          _stream(stream, phi.device))
