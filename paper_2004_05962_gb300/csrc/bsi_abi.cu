@@ -515,6 +515,19 @@ static void split_tile_planes(InstDesc& d, int warp_smem) {
     d.units *= d.zparts;
 }
 
+// The resampling's units: strips of resample_strip_tiles tiles (a tile-config entry
+// may fix them), tile-planes split by resample_zparts.
+static void plan_resample(InstDesc& d, int buf_bytes, bool grad) {
+    if (d.units <= 0) return;
+    if (lookup_config(d.dx, d.dy, d.dz).fwd_strip_tiles == 0) d.gcells = resample_strip_tiles(d.ncx, d.dx, grad);
+    d.nxg = (int)cdiv(d.ncx, d.gcells);
+    d.units = (long long)d.ncz * d.ncy * d.nxg;
+    const int wsm = resample_warp_smem(buf_bytes), wpc = warps_per_cta(wsm, d.warps_req);
+    const int ctas = imax(1, imin(3, kTmaSmemBudget / (wpc * wsm + 1024)));
+    d.zparts = resample_zparts(d.units, (long long)device_sms() * ctas * wpc, d.dz, d.dy);
+    d.units *= d.zparts;
+}
+
 enum class Op { Forward, AdjointPartials, AdjointReduce };
 
 template <int MAXB>
@@ -859,10 +872,13 @@ static void check_cells(const RatDesc& d, const CellPlan& c, bool adjoint, Range
         }
 }
 
-static void check_forward_group(Group g, int ob, RangeChecker& rc, bool cover, bool split) {
+// split: the units a call of one volume takes (0: whole tile-planes, 1: forward, 2 / 3:
+// resampling value / gradient mode).
+static void check_forward_group(Group g, int ob, RangeChecker& rc, bool cover, int split) {
     const int buf = stage_buf_bytes(g.dxmax);
     for (InstDesc& d : g.inst) {
-        if (split) split_tile_planes(d, fwd_warp_smem(buf));
+        if (split == 1) split_tile_planes(d, fwd_warp_smem(buf));
+        else if (split > 1) plan_resample(d, buf, split == 3);
         const long long phi_elems = 3LL * d.nx * d.ny * d.nz;
         const long long nvox_all = (long long)d.X * d.Y * d.Z;
         std::vector<unsigned char> hit(cover ? (size_t)d.X * d.Y * d.Z : 0, 0);
@@ -1063,6 +1079,8 @@ static bsi_status run_resample(const bsi_geom* g, const float* phi, const float*
     grp.inst.push_back(d);
     Batch<1> b;
     to_batch(grp, b);
+    plan_resample(b.inst[0], b.buf_bytes, grad);
+    b.total_units = b.inst[0].units;
     (void)cudaGetLastError();
     const cudaError_t e = launch_resample(b, grad, grp.generic, s, nullptr);
     return e == cudaSuccess ? BSI_OK : cuda_fail(e);
@@ -1472,7 +1490,7 @@ int bsi_selfcheck_ranges(const bsi_instance* inst, int n, int op, int cover, cha
             for (const Group& g : plan(all, nullptr)) {
                 // staging bytes per voxel: the field (12 FP32, 6 BF16), T for both
                 // resampling modes (12), the scalar forward (4 FP32, 2 BF16)
-                check_forward_group(g, op == 1 ? 6 : op == 5 ? 4 : op == 6 ? 2 : 12, rc, cover != 0, n == 1 && op != 3 && op != 4);
+                check_forward_group(g, op == 1 ? 6 : op == 5 ? 4 : op == 6 ? 2 : 12, rc, cover != 0, n != 1 ? 0 : op == 3 || op == 4 ? op - 1 : 1);
                 // the single-volume forward's tensor-store path (3 or 1 channels)
                 if ((op == 0 || op == 1 || op == 5 || op == 6) && n == 1 && g.inst.size() == 1 && !g.generic)
                     check_forward_tma(g.inst[0], op == 1 || op == 6, op >= 5 ? 1 : 3, rc);

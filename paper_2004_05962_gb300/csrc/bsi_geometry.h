@@ -145,6 +145,11 @@ BSI_HD int fwd_strip_tiles(int X, int dx, bool bf16) {
     return kGroupCells;
 }
 
+// Shared memory of one warp of the resampling: its lanes' control points, then a
+// staging row.
+constexpr int kPhBytes = 48 * kLanes * 4;
+BSI_HD int resample_warp_smem(int buf_bytes) { return kPhBytes + buf_bytes; }
+
 // Units per tile-plane of a strip, one volume of `units` whole ones on `slots`
 // resident warps: a volume of fewer strips than warps is bound by the serial walk
 // of a unit's dy dz rows, not by bandwidth, and its tile-planes are split so that
@@ -157,6 +162,47 @@ BSI_HD int fwd_zparts(long long units, long long slots, int dz) {
     if (units <= 0 || units >= slots) return 1;
     const long long p = slots / units;
     return p < dz ? (int)p : dz;
+}
+
+// Tiles per strip of the resampling.  Its rows are sampled 32 voxels at a time, so a
+// strip of 29 tiles that ends just past such a run wastes most of one, and most of
+// all in gradient mode, which keeps one sample per lane in flight: there, and at
+// x-spacing 8 (232 voxels: 7 runs and 8 voxels), strips of equal width of at most 128
+// voxels, unless they are more than half as many again (each costs its z and y
+// stages).  Measured (us, 29 tiles -> these): gradient mode and adjoint of 512 x 512 x
+// 300 at 5 942 -> 885, 192 x 192 x 160 at 5 112 -> 101, 317 x 203 x 155 at (4, 5, 7) 176 ->
+// 159, 512 x 512 x 256 at 8 1001 -> 898; value mode at 8 638 -> 524, 301 x 222 x 131 97 ->
+// 81.  Value mode at 5 and 7 keeps 29 (539 against 597, 78 against 92).  Its stores
+// are not bulk copies: the strips need not start on 16-byte boundaries (512 x 512 x
+// 256 at 3, 28 -> 29 tiles: 592 -> 569).
+inline int resample_strip_tiles(int ncx, int dx, bool grad) {
+    const int most = 128 / dx;
+    if (dx <= 4 || dx > kMaxSpecializedDx || !(grad || dx == 8)) return kGroupCells;
+    const long long wide = cdiv(ncx, kGroupCells), n = cdiv(ncx, most);
+    return 2 * n <= 3 * wide ? (int)cdiv(ncx, n) : kGroupCells;
+}
+
+// Units per tile-plane of a strip for the resampling, by a model of the rounds over
+// the resident warps (a round that is not full costs 0.75 + 0.25 x its fill, none
+// less than one) x the rows of a unit and 1.5 for its start.  Its rows cost more
+// than the forward's and its time is their latency, so a nearly empty last round
+// or a few long units decide at every size: 160 x 192 x 192 at spacing 5 in gradient
+// mode, 2496 units on 2432 warps, 103 us whole and 84 in fifths; 131 x 222 x 301 at 8
+// 153 -> 79 us (value) and 325 -> 145 (gradient); 256 x 512 x 512 at 8 851 -> 638 and 1096 ->
+// 877.  512 x 512 x 300 at 5, 6.8 rounds, 536 us whole and 596 in fifths.
+inline int resample_zparts(long long units, long long slots, int dz, int dy) {
+    int best = 1;
+    double best_t = -1;
+    for (int p = 1; p <= dz && units > 0 && slots > 0; ++p) {
+        const double n = (double)units * p / slots, full = (double)(long long)n, f = n - full;
+        const double rounds = full + (f > 1e-9 ? 0.75 + 0.25 * f : 0.0);
+        const double t = (rounds < 1.0 ? 1.0 : rounds) * ((dz + p - 1) / p * dy + 1.5);
+        if (best_t < 0 || t < best_t) {
+            best = p;
+            best_t = t;
+        }
+    }
+    return best;
 }
 
 template <bool PARTS = true>

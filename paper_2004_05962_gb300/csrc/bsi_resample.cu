@@ -28,8 +28,6 @@ static __device__ unsigned g_err;
 // conflicts).  In registers they held 48 per thread and capped the kernel at two
 // CTAs per SM; moved out, three fit, and the extra warps hide the gathers'
 // latency (value mode -17%, gradient mode -23% on a 512x512x300 volume).
-constexpr int kPhFloats = 48 * kLanes;
-constexpr int kPhBytes = kPhFloats * 4;
 __device__ __forceinline__ int ph_index(int n, int m, int c, int lane) { return ((n * 4 + m) * 3 + c) * kLanes + lane; }
 
 // F~ at (x + tx, y + ty, z + tz) and, in GRAD mode, its gradient in grad[3].
@@ -199,7 +197,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * kLanes, GRAD ? 2 : 3)
     extern __shared__ __align__(16) unsigned char rsmem[];
     const int lane = threadIdx.x & (kLanes - 1);
     const int warp = threadIdx.x >> 5;
-    unsigned char* stage = rsmem + (size_t)warp * (b.buf_bytes + kPhBytes) + kPhBytes;
+    unsigned char* stage = rsmem + (size_t)warp * resample_warp_smem(b.buf_bytes) + kPhBytes;
     const int wpc = blockDim.x >> 5;
     const InstDesc& d = b.inst[0];
     for (long long r = 0;; ++r) {
@@ -225,9 +223,9 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * kLanes, GRAD ? 2 : 3)
 template <bool GRAD, bool GENERIC>
 static cudaError_t launch_rs_t(const Batch<1>& b, cudaStream_t s, LaunchInfo* info) {
     auto kern = bsi_resample_kernel<GRAD, GENERIC>;
-    const int wpc = warps_per_cta(b.buf_bytes + kPhBytes, b.warps_req);   // control points + a staging row per warp
+    const int wpc = warps_per_cta(resample_warp_smem(b.buf_bytes), b.warps_req);
     const int threads = wpc * kLanes;
-    const int smem = wpc * (b.buf_bytes + kPhBytes);
+    const int smem = wpc * resample_warp_smem(b.buf_bytes);
     KernelFacts f;
     cudaError_t e = kernel_facts(reinterpret_cast<const void*>(kern), threads, smem, &f);
     if (e != cudaSuccess) return e;
