@@ -216,6 +216,24 @@ static bool takes_wide(const bsi_geom& g, int n) {
     return n == 1 && g.dx > kMaxSpecializedDx && g.dy * g.dz >= kWideMinRows && !empty_volume(g);
 }
 
+// Whether the FP32 forward of one volume takes the kernels on cells of any width at
+// x-spacing 8, its widest own one (same bits): they give a row's 8-voxel cells to two
+// lanes each, which pays where the volume's width fills few of the lanes of strips of
+// 29 tiles, and where unaligned rows make the strips' shared stores conflict -- but a
+// unit's start needs some rows.  Measured (us, strips -> cells): 256^3, 55% filled,
+// 44.6 -> 35.1 at (8, 8, 8), 48.1 -> 34.8 at 12 rows per cell, 61 -> 54 at 4; 317 x 203 x
+// 155, 69% and unaligned, 46.4 -> 32.6 and 46.4 -> 33.3, at 4 rows equal; 160 x 400 x 400,
+// 69% and aligned, 72 -> 61 at 64 rows, 57 against 79 at 12; 512 x 512 x 300, 74%, 133
+// against 149.
+static bool takes_cells_forward(const bsi_geom& g, int n) {
+    if (takes_wide(g, n)) return true;
+    if (n != 1 || g.dx != kMaxSpecializedDx || empty_volume(g) || lookup_config(g.dx, g.dy, g.dz).fwd_strip_tiles > 0) return false;
+    const long long ncx = cdiv(g.X, g.dx);
+    const double fill = (double)ncx / (double)(cdiv(ncx, kGroupCells) * kGroupCells);
+    const int rows = g.dy * g.dz;
+    return (rows >= 12 && fill < (g.X % 4 != 0 ? 0.72 : 0.6)) || (rows >= 48 && fill < 0.72);
+}
+
 // Whether the adjoint of one volume takes the kernels on cells of any width though
 // its x-spacing has a kernel of its own: small volumes, whose few units -- at least
 // three tile-planes each -- leave most warps idle and take the time of one unit's
@@ -632,7 +650,7 @@ static bsi_status forward_impl(const bsi_instance* inst, int n, bsi_dtype dt, cu
     if (dt != BSI_F32 && dt != BSI_BF16) return BSI_ERR_DTYPE;
     bsi_status st = check_instances(inst, n, true, false, dt);
     if (st != BSI_OK) return st;
-    if (n == 1 && dt == BSI_F32 && takes_wide(inst[0].geom, n)) {
+    if (n == 1 && dt == BSI_F32 && takes_cells_forward(inst[0].geom, n)) {
         RatDesc d = wide_desc(inst[0].geom);
         d.phi = inst[0].phi;
         d.field = static_cast<float*>(inst[0].field);
@@ -1472,7 +1490,8 @@ int bsi_selfcheck_ranges(const bsi_instance* inst, int n, int op, int cover, cha
         for (int i = 0; i < n; ++i) ok = ok && check_geom(&inst[i].geom) == BSI_OK;
         if (!ok) {
             rc.fail("invalid geometry", n, 0);
-        } else if (n == 1 && (((op == 0 || op == 2) && takes_wide(inst[0].geom, n)) || (op == 2 && takes_small(inst[0].geom, n)))) {
+        } else if (n == 1 && ((op == 0 && takes_cells_forward(inst[0].geom, n)) ||
+                              (op == 2 && (takes_wide(inst[0].geom, n) || takes_small(inst[0].geom, n))))) {
             // cells of any width, for aligned and unaligned arrays
             const RatDesc d = wide_desc(inst[0].geom);
             const long long bound = adj_floats_bound(inst[0].geom);
