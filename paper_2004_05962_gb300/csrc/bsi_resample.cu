@@ -230,8 +230,14 @@ static cudaError_t launch_rs_t(const Batch<1>& b, cudaStream_t s, LaunchInfo* in
     cudaError_t e = kernel_facts(reinterpret_cast<const void*>(kern), threads, smem, &f);
     if (e != cudaSuccess) return e;
     const long long want = cdiv(b.total_units, wpc);
+    // value mode from four rounds on: a CTA per eight units, handed out as CTAs finish,
+    // which evens out the strips' unequal widths (512 x 512 x 300 at spacing 5, 6.8 rounds:
+    // 539 -> 496 us; 512 x 512 x 256 at 8, 9 rounds: 525 -> 487; 192 x 192 x 160 at 5, 3.4
+    // rounds, equal alone and 3% slower before a gradient call).  Gradient mode, whose
+    // strips are even, keeps the persistent grid (886 against 910 us)
     const long long cap = (long long)f.sms * f.ctas_per_sm;
-    const int grid = (int)(want < cap ? want : cap);
+    const long long all = want < 0x7fffffffLL ? want : 0x7fffffffLL;
+    const int grid = (int)(!GRAD && want >= 4 * cap ? all : want < cap ? want : cap);
     if (info) *info = LaunchInfo{grid, threads, smem, f.ctas_per_sm};
     if (grid <= 0) return cudaSuccess;
     kern<<<grid, threads, smem, s>>>(b);
