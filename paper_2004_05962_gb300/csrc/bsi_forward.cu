@@ -68,8 +68,13 @@ static cudaError_t launch_fwd_t(const Batch<MAXB>& b, cudaStream_t s, LaunchInfo
     KernelFacts f;
     cudaError_t e = kernel_facts(reinterpret_cast<const void*>(kern), threads, smem, &f);
     if (e != cudaSuccess) return e;
+    // More CTAs than are resident, so that SMs that finish early take more, where units are
+    // uneven or short: batches 2x (64 volumes: 443 -> 426 us; 4x 432, all units' CTAs 487),
+    // unaligned rows 2x (317 x 203 x 155 at (4, 5, 7): 27.5 -> 26.1), one channel 4x (4x zoom
+    // to 512 x 512 x 300: 70.1 -> 67.8).  Aligned FP32 rows gain nothing (512 x 512 x 300 at
+    // 5: 135.6, 136.7 at 2x) and keep the grid that is wholly resident.
     const long long want = cdiv(b.total_units, wpc);
-    const long long cap = (long long)f.sms * f.ctas_per_sm;
+    const long long cap = (long long)f.sms * f.ctas_per_sm * (C == 1 ? 4 : MAXB > 1 || b.inst[0].X % 4 != 0 ? 2 : 1);
     const int grid = (int)(want < cap ? want : cap);
     if (info) *info = LaunchInfo{grid, threads, smem, f.ctas_per_sm};
     if (grid <= 0) return cudaSuccess;
