@@ -68,13 +68,15 @@ static cudaError_t launch_fwd_t(const Batch<MAXB>& b, cudaStream_t s, LaunchInfo
     KernelFacts f;
     cudaError_t e = kernel_facts(reinterpret_cast<const void*>(kern), threads, smem, &f);
     if (e != cudaSuccess) return e;
-    // More CTAs than are resident, so that SMs that finish early take more, where units are
-    // uneven or short: batches 2x (64 volumes: 443 -> 426 us; 4x 432, all units' CTAs 487),
-    // unaligned rows 2x (317 x 203 x 155 at (4, 5, 7): 27.5 -> 26.1), one channel 4x (4x zoom
-    // to 512 x 512 x 300: 70.1 -> 67.8).  Aligned FP32 rows gain nothing (512 x 512 x 300 at
-    // 5: 135.6, 136.7 at 2x) and keep the grid that is wholly resident.
+    // From eight rounds on more CTAs than are resident, so that SMs that finish early take
+    // more, where units are uneven or short: batches 2x (64 volumes: 443 -> 426 us; 4x 432,
+    // all units' CTAs 487), one channel 4x (4x zoom to 512 x 512 x 300, 20 rounds: 70.1 -> 67.8).
+    // With fewer rounds it costs more than it evens out (400 x 256 x 256 at 5, 3.3 rounds, one
+    // channel: 26.0 against 27.6); aligned FP32 rows gain nothing (512 x 512 x 300 at 5: 135.6,
+    // 136.7 at 2x).
     const long long want = cdiv(b.total_units, wpc);
-    const long long cap = (long long)f.sms * f.ctas_per_sm * (C == 1 ? 4 : MAXB > 1 || b.inst[0].X % 4 != 0 ? 2 : 1);
+    const long long resident = (long long)f.sms * f.ctas_per_sm;
+    const long long cap = resident * (want < 8 * resident ? 1 : C == 1 ? 4 : MAXB > 1 ? 2 : 1);
     const int grid = (int)(want < cap ? want : cap);
     if (info) *info = LaunchInfo{grid, threads, smem, f.ctas_per_sm};
     if (grid <= 0) return cudaSuccess;
@@ -91,7 +93,7 @@ cudaError_t launch_forward(const Batch<MAXB>& b, bool bf16, bool generic, cudaSt
 // Forward on the tensor-store path (one volume, C = 3 or 1 channels; see
 // fwd_tma_rows): the same persistent unit walk as bsi_forward_kernel, rows
 // leaving in blocks of rb.
-template <bool BF16, int C>
+template <bool BF16, int C, bool PARTS>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * kLanes, 2)
     bsi_forward_tma_kernel(const __grid_constant__ Batch<1> b, const __grid_constant__ CUtensorMap map, int rb,
                            int blk_bytes) {
@@ -109,14 +111,14 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * kLanes, 2)
         const long long ul = slot_unit(r, blockIdx.x, warp, gridDim.x, wpc, b.total_units, false);
         if (ul < 0) break;
         switch (d.dx) {
-            case 1: forward_unit_tma<1, BF16, C>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
-            case 2: forward_unit_tma<2, BF16, C>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
-            case 3: forward_unit_tma<3, BF16, C>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
-            case 4: forward_unit_tma<4, BF16, C>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
-            case 5: forward_unit_tma<5, BF16, C>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
-            case 6: forward_unit_tma<6, BF16, C>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
-            case 7: forward_unit_tma<7, BF16, C>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
-            default: forward_unit_tma<8, BF16, C>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
+            case 1: forward_unit_tma<1, BF16, C, PARTS>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
+            case 2: forward_unit_tma<2, BF16, C, PARTS>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
+            case 3: forward_unit_tma<3, BF16, C, PARTS>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
+            case 4: forward_unit_tma<4, BF16, C, PARTS>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
+            case 5: forward_unit_tma<5, BF16, C, PARTS>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
+            case 6: forward_unit_tma<6, BF16, C, PARTS>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
+            case 7: forward_unit_tma<7, BF16, C, PARTS>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
+            default: forward_unit_tma<8, BF16, C, PARTS>(d, &map, ul, stage, blk_bytes, rb, lane, ring, &g_err); break;
         }
     }
     // the blocks must outlive every tensor store that reads them
@@ -125,7 +127,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * kLanes, 2)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-template <bool BF16, int C>
+template <bool BF16, int C, bool PARTS>
 static cudaError_t launch_fwd_tma_t(const Batch<1>& b, const CUtensorMap& map, int rb, cudaStream_t s,
                                     LaunchInfo* info) {
     const InstDesc& d = b.inst[0];
@@ -134,7 +136,7 @@ static cudaError_t launch_fwd_tma_t(const Batch<1>& b, const CUtensorMap& map, i
     const int wpc = warps_per_cta(wsm, b.warps_req);
     const int threads = wpc * kLanes;
     const int smem = wpc * wsm + 128;
-    const void* kern = reinterpret_cast<const void*>(bsi_forward_tma_kernel<BF16, C>);
+    const void* kern = reinterpret_cast<const void*>(bsi_forward_tma_kernel<BF16, C, PARTS>);
     KernelFacts f;
     cudaError_t e = kernel_facts(kern, threads, smem, &f);
     if (e != cudaSuccess) return e;
@@ -143,26 +145,33 @@ static cudaError_t launch_fwd_tma_t(const Batch<1>& b, const CUtensorMap& map, i
     const int grid = (int)(want < cap ? want : cap);
     if (info) *info = LaunchInfo{grid, threads, smem, f.ctas_per_sm};
     if (grid <= 0) return cudaSuccess;
-    return launch_pdl(bsi_forward_tma_kernel<BF16, C>, grid, threads, smem, s, b, map, rb, blk_bytes);
+    return launch_pdl(bsi_forward_tma_kernel<BF16, C, PARTS>, grid, threads, smem, s, b, map, rb, blk_bytes);
 }
 
 cudaError_t launch_forward_tma(const Batch<1>& b, bool bf16, int channels, const CUtensorMap& map, int rb,
                                cudaStream_t s, LaunchInfo* info) {
+    // FP32 units of whole tile-planes, and BF16 ones at x-spacings <= 2, have kernels of their
+    // own: finding a unit's part costs units of few rows up to 4% (512 x 512 x 300 at spacing
+    // 2 419 against 437 us, at 3 204.4 against 207.9; one channel zoomed by 2 324 against 339,
+    // BF16 337 against 347).  BF16 at 5 runs 132 us with it and 135 without.
+    if (b.inst[0].zparts > 1 || (bf16 && b.inst[0].dx > 2)) {
+        if (channels == 1)
+            return bf16 ? launch_fwd_tma_t<true, 1, true>(b, map, rb, s, info) : launch_fwd_tma_t<false, 1, true>(b, map, rb, s, info);
+        return bf16 ? launch_fwd_tma_t<true, 3, true>(b, map, rb, s, info) : launch_fwd_tma_t<false, 3, true>(b, map, rb, s, info);
+    }
     if (channels == 1)
-        return bf16 ? launch_fwd_tma_t<true, 1>(b, map, rb, s, info) : launch_fwd_tma_t<false, 1>(b, map, rb, s, info);
-    return bf16 ? launch_fwd_tma_t<true, 3>(b, map, rb, s, info) : launch_fwd_tma_t<false, 3>(b, map, rb, s, info);
+        return bf16 ? launch_fwd_tma_t<true, 1, false>(b, map, rb, s, info) : launch_fwd_tma_t<false, 1, false>(b, map, rb, s, info);
+    return bf16 ? launch_fwd_tma_t<true, 3, false>(b, map, rb, s, info) : launch_fwd_tma_t<false, 3, false>(b, map, rb, s, info);
 }
 
-// Scalar (one-channel) interpolation of a single volume.  FP32 units of whole
-// tile-planes have a kernel of their own: finding a unit's part costs the large
-// ones, a few rows each, 1.4% (4x zoom to 512 x 512 x 300 70.1 against 71.1 us); no
-// other kernel shows it.
+// Scalar (one-channel) interpolation of a single volume.
 cudaError_t launch_forward_scalar(const Batch<1>& b, bool bf16, bool generic, cudaStream_t s, LaunchInfo* info) {
+    // as in launch_forward_tma (4x zoom to 512 x 512 x 300 70.1 against 71.1 us; BF16 at 5
+    // 103.9 us with parts, 105.9 without; three channels at 5 equal)
+    if (!generic && !bf16 && b.inst[0].zparts <= 1) return launch_fwd_t<1, false, false, 1, false>(b, s, info);
     if (bf16)
         return generic ? launch_fwd_t<1, true, true, 1>(b, s, info) : launch_fwd_t<1, true, false, 1>(b, s, info);
-    if (generic) return launch_fwd_t<1, false, true, 1>(b, s, info);
-    return b.inst[0].zparts > 1 ? launch_fwd_t<1, false, false, 1>(b, s, info)
-                                : launch_fwd_t<1, false, false, 1, false>(b, s, info);
+    return generic ? launch_fwd_t<1, false, true, 1>(b, s, info) : launch_fwd_t<1, false, false, 1>(b, s, info);
 }
 
 template cudaError_t launch_forward<1>(const Batch<1>&, bool, bool, cudaStream_t, LaunchInfo*);

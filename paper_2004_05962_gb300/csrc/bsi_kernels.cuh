@@ -410,7 +410,7 @@ __device__ __forceinline__ void forward_unit(const InstDesc& d, long long ul, un
 // columns past the volume's end are clipped by the copy.  Halo lanes (lane >=
 // gcells) stage into the warp's spare slot after the ring.  C = 3 channels
 // (the displacement field) or 1 (scalar interpolation).
-template <int DX, bool BF16, int C = 3>
+template <int DX, bool BF16, int C = 3, bool PARTS = true>
 __device__ __forceinline__ void forward_unit_tma(const InstDesc& d, const void* tmap, long long ul,
                                                  unsigned char* stage, int blk_bytes, int rb, int lane, int& ring,
                                                  unsigned* err) {
@@ -418,7 +418,7 @@ __device__ __forceinline__ void forward_unit_tma(const InstDesc& d, const void* 
     constexpr int ES = BF16 ? 2 : 4;
     constexpr bool PK = fwd_packed<DX, BF16>();
     constexpr int VW = BF16 ? 1 : tile_vec<DX>();
-    const FwdUnit u = fwd_unit(d, ul);
+    const FwdUnit u = fwd_unit<PARTS>(d, ul);
     const int col = u.cell0 + lane;
     float ph[4][4][C];
 #pragma unroll
