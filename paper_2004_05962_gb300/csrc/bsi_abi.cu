@@ -993,7 +993,9 @@ static void check_adjoint_group(const Group& g, long long ws_floats, RangeChecke
                     // group of the tile's last float
                     if (nv < d.dx && (xl + nv != u.nvox || d.dx - nv > d.dx - 1)) rc.fail("cut tile does not end at the row end", xl + nv, u.nvox);
                     if (12 * (xl + d.dx) + 15 > slot) rc.fail("tile past its staged row", xl, slot);
-                    if (nv < d.dx && 15 + 12 * u.nvox + 12 * (d.dx - 1) > slot) rc.fail("zeroed tail overflow", u.nvox, slot);
+                    const int missing = row_tail_voxels(d);
+                    if (nv < d.dx && (nv + missing != d.dx || 3 * missing > kLanes)) rc.fail("zeroed tail of another length", nv, missing);
+                    if (nv < d.dx && 15 + 12 * (u.nvox + missing) > slot) rc.fail("zeroed tail overflow", u.nvox, slot);
                 }
                 const int j = lane - kHalo;
                 if (j < 0 || u.col0 + j >= d.nx) continue;

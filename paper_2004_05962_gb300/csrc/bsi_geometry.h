@@ -296,6 +296,10 @@ constexpr int kRowStageBytes = 9472;
 BSI_HD int fwd_warp_smem(int buf_bytes) { return kStoreStages * buf_bytes; }
 BSI_HD int adj_warp_smem(int stage_bytes) { return kRowHeadBytes + kLoadStages * stage_bytes; }
 BSI_HD int row_stage_bytes(int dxmax) { return imax(kRowStageBytes, stage_buf_bytes(dxmax)); }
+// Zero voxels written after a staged row for the tile that the volume's end cuts:
+// what that tile lacks and no more.  Where it is the last of a strip of 32 tiles it
+// ends with the row's slot, and the next row's slot follows.
+BSI_HD int row_tail_voxels(const InstDesc& d) { return d.ncx * d.dx - d.X; }
 // Rows per block at spacing (dx, dy): as many as fit a stage, in even blocks.
 BSI_HD int row_block_rows(int dx, int dy) {
     const int rb = imax(1, imin(imin(dy, kLanes), kRowStageBytes / stage_buf_bytes(dx)));

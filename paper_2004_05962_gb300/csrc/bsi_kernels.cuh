@@ -654,7 +654,8 @@ __device__ __forceinline__ void gather_tile_phase(float (&q4)[4][3], uint32_t sv
 // 0.523 ms, now 0.411; 255 x 256 x 256 at spacing 8 0.165 -> 0.110, at 4 0.081 ->
 // 0.059, at 5 0.057 -> 0.050 ms).  Two stages of 9.25 KB; three of 6.2 KB made the
 // batch 0.50 ms.  Empty tiles read the warp's spare
-// zeros; a tile cut by the volume's end reads zeros written after its row.
+// zeros; a tile cut by the volume's end reads zeros written after its row, inside
+// the row's slot.
 template <int DX>
 __device__ __forceinline__ bool adjoint_unit(const InstDesc& d, long long ul, uint64_t* bars, uint32_t spare,
                                              unsigned char* ring, int stage_bytes, int lane, unsigned& q,
@@ -665,9 +666,9 @@ __device__ __forceinline__ bool adjoint_unit(const InstDesc& d, long long ul, ui
     const int nv = (cell >= 0 && cell < d.ncx) ? imin(dx, d.X - cell * dx) : 0;
     const int slot = stage_buf_bytes(dx), rb = d.row_block;
     // A specialised spacing reads all DX voxels of every lane, unpredicated: the
-    // missing voxels of a cut tile are the zeros after the row's nvox voxels.
+    // missing voxels of a cut tile are zeros after the row's nvox voxels.
     const bool cut = DX > 0 && __any_sync(kFull, nv > 0 && nv < dx);
-    const int zfloats = 3 * (dx - 1);
+    const int zfloats = 3 * row_tail_voxels(d);
     const int y0 = u.jy * d.dy, yn = imin(d.dy, d.Y - y0);
     const int nblk = (yn + rb - 1) / rb;
     const int zb = u.kz0 * d.dz;
