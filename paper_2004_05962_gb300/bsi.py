@@ -221,12 +221,19 @@ def _ints(values):
     return tuple(map(int, values))
 
 
+# The raw handle of a device's current stream (a Stream object takes 2 us to make); not
+# part of torch's documented interface, so the documented call stands in where it is missing.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream, device) -> int:
-    if stream is None:
-        # (the raw handle: a Stream object takes 2 us to make)
-        return torch._C._cuda_getCurrentRawStream(device.index) if device is not None and device.index is not None \
-            else torch.cuda.current_stream(device).cuda_stream
-    return int(stream.cuda_stream)
+    """The handle of ``stream``, or of the current stream of ``device``: a CUDA tensor's
+    device, or whatever torch.cuda.current_stream takes."""
+    if stream is not None:
+        return int(stream.cuda_stream)
+    if _raw_stream is not None and isinstance(device, torch.device) and device.type == "cuda" and device.index is not None:
+        return _raw_stream(device.index)
+    return torch.cuda.current_stream(device).cuda_stream
 
 
 def _check(st, where):
