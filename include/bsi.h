@@ -191,7 +191,11 @@ bsi_status bsi_field_adjoint_noalloc(const bsi_geom* g, const float* grad_field,
 /* Launch shape for one spacing class, chosen by the autotuner
  * (paper_2004_05962_gb300/tune.py times candidates and keeps a JSON cache).
  * The paper tunes its block shape per GPU by hand (Sec. 3.4); here the shape
- * is data.  A zero field means "library default". */
+ * is data.  A zero field means "library default"; that covers the kernels
+ * without these shapes (x-cells of any width) which one volume may take at
+ * dx <= 8: a non-zero field of a direction keeps its calls on the kernels that
+ * the field shapes.  At dx > 8 with dy * dz >= 16 the FP32 forward and the
+ * adjoint of one volume take the former whatever the entry says. */
 typedef struct {
     int32_t dx, dy, dz;        /* spacing the entry applies to; 0 matches any value */
     int32_t adj_zchunk;        /* adjoint: tile-planes per warp unit, 3..16 (0: chosen per volume

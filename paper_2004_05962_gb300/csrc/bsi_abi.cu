@@ -210,7 +210,8 @@ static RatDesc wide_desc(const bsi_geom& g) {
 // Whether a call over n volumes takes those kernels (g: the only volume): their
 // unit is a z-cell or a part of one, whose start is worth it from about 16 rows
 // on (forward + adjoint of 256^3 at 12: 0.405 -> 0.117 ms, at 20: 1.395 -> 0.118
-// ms; 250 x 256 x 200 at (9, 3, 3), 9 rows: 0.093 against 0.113 ms).
+// ms; 250 x 256 x 200 at (9, 3, 3), 9 rows: 0.093 against 0.113 ms).  They have
+// none of the shapes of the tile-config table.
 constexpr int kWideMinRows = 16;
 static bool takes_wide(const bsi_geom& g, int n) {
     return n == 1 && g.dx > kMaxSpecializedDx && g.dy * g.dz >= kWideMinRows && !empty_volume(g);
@@ -225,9 +226,12 @@ static bool takes_wide(const bsi_geom& g, int n) {
 // 155, 69% and unaligned, 46.4 -> 32.6 and 46.4 -> 33.3, at 4 rows equal; 160 x 400 x 400,
 // 69% and aligned, 72 -> 61 at 64 rows, 57 against 79 at 12; 512 x 512 x 300, 74%, 133
 // against 149.
+// A tile-config entry that shapes the strips' launch keeps them.
 static bool takes_cells_forward(const bsi_geom& g, int n) {
     if (takes_wide(g, n)) return true;
-    if (n != 1 || g.dx != kMaxSpecializedDx || empty_volume(g) || lookup_config(g.dx, g.dy, g.dz).fwd_strip_tiles > 0) return false;
+    if (n != 1 || g.dx != kMaxSpecializedDx || empty_volume(g)) return false;
+    const bsi_tile_config cfg = lookup_config(g.dx, g.dy, g.dz);
+    if (cfg.fwd_strip_tiles > 0 || cfg.fwd_warps > 0) return false;
     const long long ncx = cdiv(g.X, g.dx);
     const double fill = (double)ncx / (double)(cdiv(ncx, kGroupCells) * kGroupCells);
     const int rows = g.dy * g.dz;
@@ -245,11 +249,13 @@ static bool takes_cells_forward(const bsi_geom& g, int n) {
 // (192 x 192 x 160 at 3, 27 rows: 26.3 against 36.9), unless most warps idle (64^3 at
 // 3: 14.1 -> 11.8).  A rule of the geometry only (a 152-SM GPU, 16-byte-aligned
 // gradient), so that a workspace query knows the answer; a tile-config entry that
-// fixes the tile-planes per unit keeps them.
+// shapes the units' launch keeps them.
 constexpr double kSmallFill = 0.65, kSmallAnyFill = 0.3;
 constexpr int kSmallRows = 48;
 static bool takes_small(const bsi_geom& g, int n) {
-    if (n != 1 || empty_volume(g) || g.dx > kMaxSpecializedDx || lookup_config(g.dx, g.dy, g.dz).adj_zchunk > 0) return false;
+    if (n != 1 || empty_volume(g) || g.dx > kMaxSpecializedDx) return false;
+    const bsi_tile_config cfg = lookup_config(g.dx, g.dy, g.dz);
+    if (cfg.adj_zchunk > 0 || cfg.adj_warps > 0) return false;
     InstDesc d;
     fill_desc(d, g, true);
     const bool tma = d.X % 4 == 0;
