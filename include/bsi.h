@@ -98,7 +98,10 @@ bsi_status bsi_field_forward(const bsi_geom* g, const float* phi, void* field, b
  * volume); no counterpart in the paper (its kernels have no adjoint): the
  * most any of its launch plans can use, since the tile-planes (and, on the
  * tensor-copy path, tile-rows) per warp unit are chosen per call (from the
- * device's SM count) unless the tile-config table fixes the tile-planes. */
+ * device's SM count) unless the tile-config table fixes the tile-planes.
+ * Volumes too small to fill the GPU with such units, and x-spacings above 8,
+ * take smaller units, with more partial sums (256^3 at spacing 12: 10.4 MB,
+ * where units of tile-planes need 1.5 MB; 64^3 at 5: 2.1 and 0.5 MB). */
 size_t bsi_adjoint_workspace_bytes(const bsi_geom* g);
 
 /* Adjoint BSI: the transpose of Eq. 1 applied to a voxel gradient,
@@ -142,8 +145,9 @@ bsi_status bsi_field_forward_batched(const bsi_instance* inst, int n, bsi_dtype 
                                      bsi_stream_t stream);
 
 /* Workspace bytes bsi_field_adjoint_batched needs for these n instances (no
- * counterpart in the paper): the sum of each instance's bound, 16-byte aligned
- * per instance. */
+ * counterpart in the paper): the sum of each instance's bound over units of
+ * tile-planes, 16-byte aligned per instance; for n == 1, the bytes of
+ * bsi_adjoint_workspace_bytes. */
 size_t bsi_batched_adjoint_workspace_bytes(const bsi_instance* inst, int n);
 
 /* Batched adjoint over n volumes (no counterpart in the paper): the transpose

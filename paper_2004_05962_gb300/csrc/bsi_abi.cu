@@ -274,8 +274,9 @@ static bool takes_small(const bsi_geom& g, int n) {
 // Workspace floats an adjoint instance may need: the most (least, with
 // `least`) over every plan the launch may pick -- tile-rows per unit 1, or also
 // kTmaJrows where the volume could take the tensor-copy path, times the table's
-// zchunk if it fixes one, else every zchunk choose_zchunk may pick.
-static long long adj_floats_bound(const bsi_geom& g, bool least = false) {
+// zchunk if it fixes one, else every zchunk choose_zchunk may pick -- and, in a call
+// of one volume (n == 1), the cells kernels' plans where it takes those.
+static long long adj_floats_bound(const bsi_geom& g, int n, bool least = false) {
     InstDesc d;
     fill_desc(d, g, true);
     const bool fixed = lookup_config(g.dx, g.dy, g.dz).adj_zchunk > 0;
@@ -291,7 +292,7 @@ static long long adj_floats_bound(const bsi_geom& g, bool least = false) {
             if (fixed) break;
         }
     }
-    if (!least && (takes_wide(g, 1) || takes_small(g, 1)))
+    if (!least && (takes_wide(g, n) || takes_small(g, n)))
         m = std::max(m, std::max(cell_plan(wide_desc(g), true, false).part_floats, cell_plan(wide_desc(g), true, true).part_floats));
     return m;
 }
@@ -683,7 +684,7 @@ static bsi_status adjoint_impl(const bsi_instance* inst, int n, void* ws, size_t
         const RatDesc d = wide_desc(inst[0].geom);
         const long long have = (long long)(ws_bytes / sizeof(float));
         const CellPlan c = cell_plan(d, true, !misaligned(inst[0].grad_field, 16), fixed_scratch ? have : -1);
-        if (!fixed_scratch && adj_floats_bound(inst[0].geom) > have) return BSI_ERR_WORKSPACE;
+        if (!fixed_scratch && adj_floats_bound(inst[0].geom, n) > have) return BSI_ERR_WORKSPACE;
         if (c.part_floats <= have) {   // else (fixed scratch): the plans below have smaller ones
             if (!ws) return BSI_ERR_WORKSPACE;
             if (misaligned(ws, 16)) return BSI_ERR_ALIGN;
@@ -701,7 +702,7 @@ static bsi_status adjoint_impl(const bsi_instance* inst, int n, void* ws, size_t
     // the documented size (the bound over zchunk choices), not only this plan's
     long long bound = 0;
     if (!fixed_scratch)
-        for (int i = 0; i < n; ++i) bound += adj_floats_bound(inst[i].geom);
+        for (int i = 0; i < n; ++i) bound += adj_floats_bound(inst[i].geom, n);
     if ((size_t)std::max(bound, ws_floats) * sizeof(float) > ws_bytes) return BSI_ERR_WORKSPACE;
     if (ws_floats > 0 && !ws) return BSI_ERR_WORKSPACE;
     if (ws && misaligned(ws, 16)) return BSI_ERR_ALIGN;
@@ -1058,12 +1059,12 @@ static void check_adjoint_plans(const bsi_instance* inst, int n, bool cover, Ran
     const std::vector<Group> groups = plan(descs(inst, n, true, false, true), &ws, true);
     // the documented workspace (the bound over every plan) holds the planned one
     long long bound = 0;
-    for (int i = 0; i < n; ++i) bound += adj_floats_bound(inst[i].geom);
+    for (int i = 0; i < n; ++i) bound += adj_floats_bound(inst[i].geom, n);
     if (ws > bound) rc.fail("planned workspace over the documented bound", ws, bound);
     // and so does the least bound the no-alloc entry point admits a volume by
     if (n == 1) {
         long long ws1 = 0;
-        const long long least = adj_floats_bound(inst[0].geom, true);
+        const long long least = adj_floats_bound(inst[0].geom, 1, true);
         (void)plan(descs(inst, 1, true, false, true, least), &ws1, true);
         if (ws1 > least) rc.fail("no plan fits the least bound", ws1, least);
     }
@@ -1178,7 +1179,7 @@ bsi_status bsi_field_forward(const bsi_geom* g, const float* phi, void* field, b
 
 size_t bsi_adjoint_workspace_bytes(const bsi_geom* g) {
     if (check_geom(g) != BSI_OK) return 0;
-    return (size_t)adj_floats_bound(*g) * sizeof(float);
+    return (size_t)adj_floats_bound(*g, 1) * sizeof(float);
 }
 
 bsi_status bsi_field_adjoint(const bsi_geom* g, const float* grad_field, float* grad_phi, void* workspace,
@@ -1201,7 +1202,7 @@ size_t bsi_batched_adjoint_workspace_bytes(const bsi_instance* inst, int n) {
     long long total = 0;
     for (int i = 0; i < n; ++i) {
         if (check_geom(&inst[i].geom) != BSI_OK) return 0;
-        total += adj_floats_bound(inst[i].geom);
+        total += adj_floats_bound(inst[i].geom, n);
     }
     return (size_t)total * sizeof(float);
 }
@@ -1443,7 +1444,7 @@ bsi_status bsi_resample_forward(const bsi_geom* g, const float* phi, const float
 
 size_t bsi_resample_backward_workspace_bytes(const bsi_geom* g) {
     if (check_geom(g) != BSI_OK || empty_volume(*g)) return 0;
-    return round256((size_t)12 * g->X * g->Y * g->Z) + (size_t)adj_floats_bound(*g) * sizeof(float);
+    return round256((size_t)12 * g->X * g->Y * g->Z) + (size_t)adj_floats_bound(*g, 1) * sizeof(float);
 }
 
 bsi_status bsi_resample_backward(const bsi_geom* g, const float* phi, const float* floating, int64_t fX, int64_t fY,
@@ -1502,7 +1503,7 @@ int bsi_selfcheck_ranges(const bsi_instance* inst, int n, int op, int cover, cha
                               (op == 2 && (takes_wide(inst[0].geom, n) || takes_small(inst[0].geom, n))))) {
             // cells of any width, for aligned and unaligned arrays
             const RatDesc d = wide_desc(inst[0].geom);
-            const long long bound = adj_floats_bound(inst[0].geom);
+            const long long bound = adj_floats_bound(inst[0].geom, n);
             for (int vec = 0; vec < 2; ++vec) {
                 const CellPlan c = cell_plan(d, op == 2, vec != 0);
                 check_cells(d, c, op == 2, rc, cover != 0);
@@ -1593,7 +1594,7 @@ extern "C" bsi_status bsi_field_adjoint_noalloc(const bsi_geom* g, const float* 
     const bsi_status st = check_instances(&in, 1, false, true, BSI_F32);
     if (st != BSI_OK) return st;
     // the smallest plan must fit; adjoint_impl then picks among the plans that do
-    const size_t need = empty_volume(*g) ? 0 : (size_t)adj_floats_bound(*g, true) * sizeof(float);
+    const size_t need = empty_volume(*g) ? 0 : (size_t)adj_floats_bound(*g, 1, true) * sizeof(float);
     if (need > kNoAllocScratchBytes) return BSI_ERR_SCRATCH_LIMIT;
     void* scratch = nullptr;
     if (need > 0) {
