@@ -406,11 +406,13 @@ bsi_status bsi_selftest_lost_copy(bsi_stream_t stream);
  * fails. */
 bsi_status bsi_probe_fill(void* dst, size_t bytes, uint32_t value, bsi_stream_t stream);
 
-/* Host-only diagnostic, no CUDA call: plans the launches of a batched call of
- * kind op (0 forward FP32, 1 forward BF16, 2 adjoint, 3 / 4 the resampling's
- * value / gradient launch, 5 / 6 the scalar forward FP32 / BF16, on each
- * instance's geometry) exactly as the entry
- * points do, and checks with the kernels' own index functions that every
+/* Host-only diagnostic, no CUDA call: plans the launches of kind op (0 forward
+ * FP32, 1 forward BF16, 2 adjoint of one call over the n instances, 3 / 4 the
+ * resampling's value / gradient launch, 5 / 6 the scalar forward FP32 / BF16, one
+ * call per instance) as the entry points do on a 152-SM GPU -- where a plan
+ * depends on the output's or, at x-spacings above 8, the gradient's alignment,
+ * for both; non-integer spacings have no op -- and checks with the kernels' own
+ * index functions that every
  * global read and write lies inside its buffer and every staging copy fits
  * its shared-memory buffer.  With cover != 0 it also checks that the forward
  * writes each voxel exactly once and that the adjoint reduce reads only

@@ -523,6 +523,12 @@ static bool bf16_odd_strips(InstDesc& d, bool bf16, bool generic) {
     return true;
 }
 
+// Scalar interpolation takes the tensor-store path where fwd_tma_rows allows it,
+// except FP32 at x-spacing 4, whose lanes store their 16-byte tiles directly
+// (4x zoom to 512 x 512 x 300: 0.070 ms direct, 0.078 ms in blocks; blocks at
+// spacing 3: 0.157 -> 0.140 ms, BF16 at 4: 0.107 -> 0.096 ms).
+static bool scalar_direct(const InstDesc& d, bool bf16) { return !bf16 && d.dx == 4; }
+
 // Rows per block when a single-volume forward of c channels takes the
 // tensor-store path, else 0.
 static int forward_tma_rows(const InstDesc& d, bool bf16, bool generic, int c = 3) {
@@ -531,9 +537,12 @@ static int forward_tma_rows(const InstDesc& d, bool bf16, bool generic, int c = 
     return fwd_tma_rows(d.X, d.dx, d.dy, d.gcells, bf16, c);
 }
 
-// Splits the tile-planes of a small volume's forward units (fwd_zparts), a warp
-// taking warp_smem bytes of shared memory, two CTAs on an SM at most.
-static void split_tile_planes(InstDesc& d, int warp_smem) {
+// Splits the tile-planes of a small volume's forward units (fwd_zparts), two CTAs
+// on an SM at most.  rb > 0: rows leave in blocks of rb (the tensor-store path),
+// else one by one through staging rows of buf_bytes.
+static void split_tile_planes(InstDesc& d, bool bf16, int c, int rb, int buf_bytes) {
+    const int warp_smem = rb > 0 ? fwd_tma_warp_smem(pad128(rb * fwd_tma_row_bytes(d.gcells, d.dx, bf16, c)))
+                                 : fwd_warp_smem(buf_bytes);
     const int wpc = warps_per_cta(warp_smem, d.warps_req);
     const int ctas = imax(1, imin(2, kTmaSmemBudget / (wpc * warp_smem + 1024)));
     d.zparts = fwd_zparts(d.units, (long long)device_sms() * ctas * wpc, d.dz);
@@ -577,8 +586,7 @@ static cudaError_t run_group(const Group& g, Op op, bool bf16, float* part, long
             const int rb = forward_tma_rows(d, bf16, g.generic);
             CUtensorMap map;
             const bool blocks = rb > 0 && encode_field_map(d, bf16, rb, &map) == cudaSuccess;
-            split_tile_planes(d, blocks ? fwd_tma_warp_smem(pad128(rb * fwd_tma_row_bytes(d.gcells, d.dx, bf16)))
-                                        : fwd_warp_smem(b.buf_bytes));
+            split_tile_planes(d, bf16, 3, blocks ? rb : 0, b.buf_bytes);
             b.total_units = d.units;
             if (blocks) return launch_forward_tma(b, bf16, 3, map, rb, s, nullptr);
             return launch_forward(b, bf16, g.generic, s, nullptr);
@@ -768,17 +776,12 @@ static void check_slots(long long total, RangeChecker& rc) {
 // the rows of the units tile the field exactly once.
 // ob: staging bytes per voxel (12 / 6 forward FP32 / BF16, 12 for T in both
 // resampling modes); outputs are checked as voxel ranges.
-// The tensor-store path of a single-volume forward (as run_group plans it for a
-// 16-byte-aligned field): every box starts on a 16-byte boundary at a
+// The tensor-store path of a single-volume forward (d: as planned for a
+// 16-byte-aligned field, rb rows per block): every box starts on a 16-byte boundary at a
 // non-negative coordinate, is at most 256 elements wide, covers exactly its
 // strip (or runs past the volume's end, where the copy clips it), stays in its
 // tile-row, and every lane's staging stays in its block row or the spare slot.
-static void check_forward_tma(const InstDesc& d0, bool bf16, int c, RangeChecker& rc) {
-    InstDesc d = d0;
-    if (c == 3) bf16_odd_strips(d, bf16, false);
-    if (c == 1 && !bf16 && d.dx == 4) return;   // direct stores (bsi_scalar_forward)
-    const int rb = fwd_tma_rows(d.X, d.dx, d.dy, d.gcells, bf16, c);
-    if (rb <= 0) return;
+static void check_forward_tma(const InstDesc& d, bool bf16, int c, int rb, RangeChecker& rc) {
     const int es = bf16 ? 2 : 4, tile = d.dx * c * es;
     const int rowb = fwd_tma_row_bytes(d.gcells, d.dx, bf16, c);
     const int blk = pad128(rb * rowb), wsm = fwd_tma_warp_smem(blk);
@@ -897,13 +900,10 @@ static void check_cells(const RatDesc& d, const CellPlan& c, bool adjoint, Range
         }
 }
 
-// split: the units a call of one volume takes (0: whole tile-planes, 1: forward, 2 / 3:
-// resampling value / gradient mode).
-static void check_forward_group(Group g, int ob, RangeChecker& rc, bool cover, int split) {
+// blocks: the rows leave in blocks, whose staging check_forward_tma checks.
+static void check_forward_group(const Group& g, int ob, RangeChecker& rc, bool cover, bool blocks = false) {
     const int buf = stage_buf_bytes(g.dxmax);
-    for (InstDesc& d : g.inst) {
-        if (split == 1) split_tile_planes(d, fwd_warp_smem(buf));
-        else if (split > 1) plan_resample(d, buf, split == 3);
+    for (const InstDesc& d : g.inst) {
         const long long phi_elems = 3LL * d.nx * d.ny * d.nz;
         const long long nvox_all = (long long)d.X * d.Y * d.Z;
         std::vector<unsigned char> hit(cover ? (size_t)d.X * d.Y * d.Z : 0, 0);
@@ -925,8 +925,8 @@ static void check_forward_group(Group g, int ob, RangeChecker& rc, bool cover, i
             if (u.rz0 < 0 || u.rz1 > d.dz) rc.fail("planes of a part", u.rz0, u.rz1);
             // a specialised spacing stages all 32 lanes x dx voxels (past the row end too)
             const int staged = d.dx <= kMaxSpecializedDx && !g.generic ? kLanes * d.dx : u.nvox;
-            if (u.nvox > staged || 15 + staged * ob > buf) rc.fail("staging overflow", staged, buf);
-            if (warps_per_cta(fwd_warp_smem(buf)) * fwd_warp_smem(buf) > kSmemBudget)
+            if (!blocks && (u.nvox > staged || 15 + staged * ob > buf)) rc.fail("staging overflow", staged, buf);
+            if (!blocks && warps_per_cta(fwd_warp_smem(buf)) * fwd_warp_smem(buf) > kSmemBudget)
                 rc.fail("forward shared memory over budget", buf, kSmemBudget);
             for (int rz = u.rz0; rz < zn; ++rz)
                 for (int ry = 0; ry < yn; ++ry) {
@@ -1073,6 +1073,43 @@ static void check_adjoint_plans(const bsi_instance* inst, int n, bool cover, Ran
         long long total = 0;
         for (const InstDesc& d : g.inst) total += d.units;
         if (cover) check_slots(total, rc);
+    }
+}
+
+// The launches of a forward, scalar forward or resampling call (op as in
+// bsi_selfcheck_ranges) that takes strips: whole tile-planes where a launch holds
+// several volumes, a lone volume's units otherwise -- for an output off and on a
+// 16-byte boundary, rows leaving in blocks there where the geometry allows it.
+static void check_forward_plans(const bsi_instance* inst, int n, int op, bool cover, RangeChecker& rc) {
+    const bool resample = op == 3 || op == 4, bf16 = op == 1 || op == 6;
+    const int c = op >= 5 ? 1 : 3;
+    // staging bytes per voxel: the field (12 FP32, 6 BF16), T for both resampling
+    // modes (12), the scalar forward (4 FP32, 2 BF16)
+    const int ob = op == 1 ? 6 : op == 5 ? 4 : op == 6 ? 2 : 12;
+    std::vector<InstDesc> all = descs(inst, n, false, bf16);
+    all.erase(std::remove_if(all.begin(), all.end(), [](const InstDesc& d) { return d.units == 0; }), all.end());
+    for (const Group& g : plan(all, nullptr)) {
+        const bool lone = g.inst.size() == 1;
+        const int buf = stage_buf_bytes(g.dxmax);
+        for (int aligned = 0; aligned < (lone && !resample ? 2 : 1); ++aligned) {
+            Group p = g;
+            InstDesc& d = p.inst[0];
+            int rb = 0;
+            if (resample) {
+                plan_resample(d, buf, op == 4);
+            } else if (lone) {
+                if (c == 3) bf16_odd_strips(d, bf16, g.generic);
+                if (aligned && !g.generic && !(c == 1 && scalar_direct(d, bf16)))
+                    rb = fwd_tma_rows(d.X, d.dx, d.dy, d.gcells, bf16, c);
+                if (aligned && rb <= 0) continue;
+                split_tile_planes(d, bf16, c, rb, buf);
+            }
+            check_forward_group(p, ob, rc, cover, rb > 0);
+            if (rb > 0) check_forward_tma(d, bf16, c, rb, rc);
+            long long total = 0;
+            for (const InstDesc& i : p.inst) total += i.units;
+            if (cover) check_slots(total, rc);
+        }
     }
 }
 
@@ -1274,12 +1311,6 @@ bsi_status bsi_check_device_status(bsi_stream_t stream, uint32_t* flags) {
     return w ? BSI_ERR_DEVICE_STATUS : BSI_OK;
 }
 
-// Scalar interpolation takes the tensor-store path where fwd_tma_rows allows it,
-// except FP32 at x-spacing 4, whose lanes store their 16-byte tiles directly
-// (4x zoom to 512 x 512 x 300: 0.070 ms direct, 0.078 ms in blocks; blocks at
-// spacing 3: 0.157 -> 0.140 ms, BF16 at 4: 0.107 -> 0.096 ms).
-constexpr bool kScalarTma = true;
-
 bsi_status bsi_scalar_forward(const bsi_geom* g, const float* coeff, void* out, bsi_dtype out_dtype,
                               bsi_stream_t stream) {
     bsi_status st = check_geom(g);
@@ -1301,11 +1332,10 @@ bsi_status bsi_scalar_forward(const bsi_geom* g, const float* coeff, void* out, 
     to_batch(grp, b);
     (void)cudaGetLastError();
     const bool bf16 = out_dtype == BSI_BF16;
-    const int rb = kScalarTma && (bf16 || b.inst[0].dx != 4) ? forward_tma_rows(b.inst[0], bf16, grp.generic, 1) : 0;
+    const int rb = scalar_direct(b.inst[0], bf16) ? 0 : forward_tma_rows(b.inst[0], bf16, grp.generic, 1);
     CUtensorMap map;
     const bool blocks = rb > 0 && encode_field_map(b.inst[0], bf16, rb, &map, 1) == cudaSuccess;
-    split_tile_planes(b.inst[0], blocks ? fwd_tma_warp_smem(pad128(rb * fwd_tma_row_bytes(b.inst[0].gcells, b.inst[0].dx, bf16, 1)))
-                                        : fwd_warp_smem(b.buf_bytes));
+    split_tile_planes(b.inst[0], bf16, 1, blocks ? rb : 0, b.buf_bytes);
     b.total_units = b.inst[0].units;
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const cudaError_t e = blocks ? launch_forward_tma(b, bf16, 1, map, rb, s, nullptr)
@@ -1482,8 +1512,8 @@ bsi_status bsi_selftest_lost_copy(bsi_stream_t stream) {
 
 int bsi_version(void) { return 100; }
 
-// Host-only: plans the launches of a batched call exactly as the entry points
-// do and checks every global and shared-memory range the kernels will touch
+// Host-only: plans the launches of a call over n volumes as the entry points do
+// (for arrays on and off 16-byte boundaries where that decides) and checks every global and shared-memory range the kernels will touch
 // (see RangeChecker).  op: 0 forward F32, 1 forward BF16, 2 adjoint, 3 / 4
 // resampling value / gradient mode (the forward's walk), 5 / 6 scalar forward
 // F32 / BF16.  With
@@ -1508,24 +1538,19 @@ int bsi_selfcheck_ranges(const bsi_instance* inst, int n, int op, int cover, cha
                 const CellPlan c = cell_plan(d, op == 2, vec != 0);
                 check_cells(d, c, op == 2, rc, cover != 0);
                 if (c.part_floats > bound) rc.fail("planned workspace over the documented bound", c.part_floats, bound);
+                if (op != 2) continue;
+                // the no-alloc entry point's plan, where its scratch holds one
+                const long long scratch = (long long)(BSI_NOALLOC_SCRATCH_BYTES / sizeof(float));
+                const CellPlan f = cell_plan(d, true, vec != 0, scratch);
+                if (f.part_floats <= scratch) check_cells(d, f, true, rc, cover != 0);
             }
-            // where the fixed scratch does not hold those, and in batches, units of tile-planes
-            if (op == 2 && takes_small(inst[0].geom, n)) check_adjoint_plans(inst, n, cover != 0, rc);
+            // where it holds none, and in batches, units of tile-planes
+            if (op == 2) check_adjoint_plans(inst, n, cover != 0, rc);
         } else if (op != 2) {
-            std::vector<InstDesc> all = descs(inst, n, false, op == 1 || op == 6);
-            all.erase(std::remove_if(all.begin(), all.end(), [](const InstDesc& d) { return d.units == 0; }),
-                      all.end());
-            for (const Group& g : plan(all, nullptr)) {
-                // staging bytes per voxel: the field (12 FP32, 6 BF16), T for both
-                // resampling modes (12), the scalar forward (4 FP32, 2 BF16)
-                check_forward_group(g, op == 1 ? 6 : op == 5 ? 4 : op == 6 ? 2 : 12, rc, cover != 0, n != 1 ? 0 : op == 3 || op == 4 ? op - 1 : 1);
-                // the single-volume forward's tensor-store path (3 or 1 channels)
-                if ((op == 0 || op == 1 || op == 5 || op == 6) && n == 1 && g.inst.size() == 1 && !g.generic)
-                    check_forward_tma(g.inst[0], op == 1 || op == 6, op >= 5 ? 1 : 3, rc);
-                long long total = 0;
-                for (const InstDesc& d : g.inst) total += d.units;
-                if (cover) check_slots(total, rc);
-            }
+            // (the resampling and the scalar forward take one volume per call)
+            if (op < 3) check_forward_plans(inst, n, op, cover != 0, rc);
+            else
+                for (int i = 0; i < n; ++i) check_forward_plans(inst + i, 1, op, cover != 0, rc);
         } else {
             check_adjoint_plans(inst, n, cover != 0, rc);
         }
