@@ -151,7 +151,6 @@ static void fill_desc(InstDesc& d, const bsi_geom& g, bool adjoint, bool bf16 = 
     } else {
         d.zchunk = zchunk;
         d.tma_rows = tma_block_rows(d.dx, d.dy);
-        d.row_block = row_block_rows(d.dx, d.dy);
         d.nxg = empty ? 0 : (int)cdiv(d.nx, kGroupCells);
         d.nzc = empty ? 0 : (int)cdiv(d.ncz, zchunk);
         d.units = (long long)d.nzc * d.ncyu * d.nxg;
@@ -369,6 +368,7 @@ struct Group {
     bool tma = false;    // adjoint tensor-copy path
     int dxmax = 1;
     int tma_stage = 0;   // tensor-copy path: bytes of one ring stage (largest block of its instances)
+    int row_stage = 0;   // row-copy path: bytes of one ring stage
     int warps_req = 0;   // smallest non-zero warps_per_cta request of its instances
     std::vector<InstDesc> inst;
 };
@@ -379,6 +379,38 @@ static bool misaligned(const void* p, uintptr_t a) { return ((uintptr_t)p & (a -
 // multiples in a 16-byte-aligned array and x-spacing <= 8.
 static bool tma_geometry_ok(const InstDesc& d) {
     return d.units > 0 && d.dx <= kMaxSpecializedDx && d.X % 4 == 0 && !misaligned(d.grad, 16);
+}
+
+// Cost of one unit: rows x (voxels per lane row + per-row work).
+static long long unit_cost(const InstDesc& d) {
+    const long long planes = d.zchunk > 0 ? (long long)d.zchunk * d.dz : d.dz;
+    return planes * d.jrows * d.dy * (d.dx + 4);
+}
+
+// The row-copy adjoint's ring of a launch of `units` units, and its instances' blocks.
+// Stages of two rows (row_stage_bytes) make a warp about 1.15 times as fast and leave
+// fewer warps resident: taken where the first warp's units, dealt round-robin from the
+// heaviest on, are the sooner done.  Measured (us, one row a stage -> two): 60 x 132 x 85
+// at (20, 5, 3), units on less than half of the warps, 41.3 -> 35.7; 256^3 at (20, 4, 3), 1.5
+// rounds instead of one, 67.4 -> 112.
+static void plan_row_stages(Group& g, long long units) {
+    auto time = [&](bool deep) {
+        const int wsm = adj_warp_smem(row_stage_bytes(g.dxmax, deep));
+        const int wpc = warps_per_cta(wsm, g.warps_req > 0 ? imin(g.warps_req, kAdjWarpsMax) : kAdjWarpsMax);
+        const int ctas = imax(1, imin(3, kTmaSmemBudget / (wpc * wsm + 1024)));
+        const long long slots = (long long)device_sms() * ctas * wpc;
+        double t = 0;
+        size_t i = 0;
+        for (long long u = 0; u < units; u += slots) {
+            while (i + 1 < g.inst.size() && g.inst[i + 1].unit_begin <= u) ++i;
+            t += (double)unit_cost(g.inst[i]);
+        }
+        return t;
+    };
+    // (the heaviest instance's planes have rows to pair)
+    const bool deep = imin(g.inst[0].dy, g.inst[0].Y) > 1 && time(true) <= 1.15 * time(false);
+    g.row_stage = row_stage_bytes(g.dxmax, deep);
+    for (InstDesc& d : g.inst) d.row_block = row_block_rows(d.dx, d.dy, row_stage_bytes(d.dx, deep));
 }
 
 // Splits instances into groups of one kernel variant, in caller order, at most
@@ -423,10 +455,6 @@ static std::vector<Group> plan(const std::vector<InstDesc>& all, long long* ws_f
     // ~ rows x (voxels per lane row + per-row work); for a batch of uneven
     // spacings it varies ~7x; measured +3% on the 64-volume batch).  Instance
     // order never changes any result.
-    auto unit_cost = [](const InstDesc& d) {
-        const long long planes = d.zchunk > 0 ? (long long)d.zchunk * d.dz : d.dz;
-        return planes * d.jrows * d.dy * (d.dx + 4);
-    };
     for (Group& g : out)
         std::stable_sort(g.inst.begin(), g.inst.end(),
                          [&](const InstDesc& a, const InstDesc& b) { return unit_cost(a) > unit_cost(b); });
@@ -438,6 +466,7 @@ static std::vector<Group> plan(const std::vector<InstDesc>& all, long long* ws_f
             ub += d.units;
             pb += (long long)d.nx * d.ny * d.nz;
         }
+        if (!g.inst.empty() && g.inst[0].zchunk > 0 && !g.tma) plan_row_stages(g, ub);
     }
     if (ws_floats) *ws_floats = off;
     return out;
@@ -447,7 +476,7 @@ template <int MAXB>
 static void to_batch(const Group& g, Batch<MAXB>& b, bool adjoint = false) {
     std::memset(&b, 0, sizeof b);
     b.n = (int)g.inst.size();
-    b.buf_bytes = g.tma ? g.tma_stage : adjoint ? row_stage_bytes(g.dxmax) : stage_buf_bytes(g.dxmax);
+    b.buf_bytes = g.tma ? g.tma_stage : adjoint ? g.row_stage : stage_buf_bytes(g.dxmax);
     b.stages = g.tma ? tma_default_stages(g.tma_stage) : 0;
     b.warps_req = g.tma ? 0 : g.warps_req;
     for (int i = 0; i < b.n; ++i) {
@@ -979,7 +1008,7 @@ static void check_adjoint_group(const Group& g, long long ws_floats, RangeChecke
             }
             // row-copy path: a bulk load covers the 16-byte-aligned superset of the row, <=
             // nbytes + 30; a block's rows fit the stage, the twelve warps' rings the SM
-            const int slot = stage_buf_bytes(d.dx), stage = row_stage_bytes(g.dxmax);
+            const int slot = stage_buf_bytes(d.dx), stage = g.row_stage;
             if (!g.tma && 30 + u.nvox * 12 > slot) rc.fail("staging overflow", u.nvox, slot);
             if (!g.tma && (d.row_block < 1 || d.row_block > kLanes || d.row_block * slot > stage))
                 rc.fail("row block over stage", d.row_block, slot);

@@ -65,7 +65,7 @@ struct InstDesc {
 template <int MAXB>
 struct Batch {
     int n;
-    int buf_bytes;          // bytes of one staging row slot (stage_buf_bytes of the largest dx)
+    int buf_bytes;          // bytes of one staging row slot (stage_buf_bytes of the largest dx); adjoint: of a ring stage
     int warps_req;          // requested warps per CTA (0: as many as shared memory allows, <= 8)
     int stages;             // adjoint tensor-copy path: ring stages per warp (else 0)
     long long total_units;
@@ -288,21 +288,26 @@ constexpr int kLoadStages = 2;    // adjoint row-copy path: ring of blocks per w
 // Shared memory of one warp: forward -- the store ring; adjoint row-copy path --
 // a head (the stages' mbarriers, then 128 bytes of zeros), then the load ring.
 // A ring stage holds a block of rows of the instance's own x-spacing; with 9.25
-// KB stages twelve warps (three 4-warp CTAs) share an SM's shared memory.  The
-// generic kernel's rows may be longer than that: one row per block there.
+// KB stages twelve warps (three 4-warp CTAs) share an SM's shared memory.  Of the
+// generic kernel's rows it may hold one only.
 constexpr int kRowSpareOff = 64;
 constexpr int kRowHeadBytes = 256;
 constexpr int kRowStageBytes = 9472;
 BSI_HD int fwd_warp_smem(int buf_bytes) { return kStoreStages * buf_bytes; }
 BSI_HD int adj_warp_smem(int stage_bytes) { return kRowHeadBytes + kLoadStages * stage_bytes; }
-BSI_HD int row_stage_bytes(int dxmax) { return imax(kRowStageBytes, stage_buf_bytes(dxmax)); }
+// Bytes of a ring stage in a launch of x-spacings up to dxmax.  deep: two rows of the
+// widest spacing at least (the generic kernel's rows of 13 and more voxels per tile),
+// where the warps that this costs are not missed (plan_row_stages).
+BSI_HD int row_stage_bytes(int dxmax, bool deep) {
+    return imax(kRowStageBytes, (deep ? 2 : 1) * stage_buf_bytes(dxmax));
+}
 // Zero voxels written after a staged row for the tile that the volume's end cuts:
 // what that tile lacks and no more.  Where it is the last of a strip of 32 tiles it
 // ends with the row's slot, and the next row's slot follows.
 BSI_HD int row_tail_voxels(const InstDesc& d) { return d.ncx * d.dx - d.X; }
 // Rows per block at spacing (dx, dy): as many as fit a stage, in even blocks.
-BSI_HD int row_block_rows(int dx, int dy) {
-    const int rb = imax(1, imin(imin(dy, kLanes), kRowStageBytes / stage_buf_bytes(dx)));
+BSI_HD int row_block_rows(int dx, int dy, int stage_bytes) {
+    const int rb = imax(1, imin(imin(dy, kLanes), stage_bytes / stage_buf_bytes(dx)));
     return (int)cdiv(dy, cdiv(dy, rb));
 }
 

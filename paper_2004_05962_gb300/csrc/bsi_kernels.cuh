@@ -630,6 +630,30 @@ __device__ __forceinline__ void accumulate_z(float (&hz)[4][NR][3], const float 
     }
 }
 
+// x-transpose of nv voxels of a tile whose width is known at run time only.  Four
+// voxels' loads are in flight together: a wide tile is one lane's serial chain.
+// Channels, not taps, are paired here: the weights come from the table by a run-time
+// index, and a pair of them would have to be put together first.  Eight volumes of 128^3
+// at spacing 20, with the stages of two rows (plan_row_stages): 1337 us with pairs of taps and one
+// voxel at a time, 795.
+__device__ __forceinline__ void gather_run_dynamic(float (&q4)[4][3], uint32_t sv, int nv, int wxb) {
+    int v = 0;
+    for (; v + 4 <= nv; v += 4) {
+        float g[12];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) g[i] = lds_f32(sv + 12u * v + 4 * i);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int l = 0; l < 4; ++l) fma3(q4[l], c_lut.w[wxb + 4 * (v + i) + l], g[3 * i], g[3 * i + 1], g[3 * i + 2]);
+    }
+    for (; v < nv; ++v) {
+        const float g0 = lds_f32(sv + 12u * v), g1 = lds_f32(sv + 12u * v + 4), g2 = lds_f32(sv + 12u * v + 8);
+#pragma unroll
+        for (int l = 0; l < 4; ++l) fma3(q4[l], c_lut.w[wxb + 4 * v + l], g0, g1, g2);
+    }
+}
+
 // x-transpose of a tile of DX voxels (DX a multiple of 4) whose row starts PH
 // floats past a 16-byte boundary, from the boundary at sv: whole 16-byte vectors,
 // the tile's values taken from them by position.  The lanes' tiles are 12 DX
@@ -798,7 +822,7 @@ __device__ __forceinline__ bool adjoint_unit(const InstDesc& d, long long ul, ui
                     } else if constexpr (DX > 0) {
                         gather_tile<DX, 1>(q4, sv + ph);
                     } else {
-                        for (int v = 0; v < nv; ++v) gather_voxel(q4, sv + ph + 12u * v, wxb + 4 * v);
+                        gather_run_dynamic(q4, sv + ph, nv, wxb);
                     }
                     sv += stride;
                     ph = (ph + (uint32_t)row_pitch) & 15u;
