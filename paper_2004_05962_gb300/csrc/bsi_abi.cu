@@ -246,11 +246,16 @@ static bool takes_cells_forward(const bsi_geom& g, int n) {
 // x 100 at (5, 5, 5) 34.6 -> 28.7.  Not where the units fill two thirds of the warps
 // (256^3 at 5: 88%, 46.3 against 51.5; 317 x 203 x 155 at 5: 74%, equal) or are short
 // (192 x 192 x 160 at 3, 27 rows: 26.3 against 36.9), unless most warps idle (64^3 at
-// 3: 14.1 -> 11.8).  A rule of the geometry only (a 152-SM GPU, 16-byte-aligned
-// gradient), so that a workspace query knows the answer; a tile-config entry that
-// shapes the units' launch keeps them.
+// 3: 14.1 -> 11.8).  Nor units of few rows in all (882 x 1 x 3 at (3, 2, 6) 6.1 against
+// 8.2; 2920 x 10 x 2 at (1, 8, 7) 7.6 against 14.6), narrow tiles from 55% on (168 x 195
+// x 278 at (4, 7, 6) 32.7 against 45.0) or short units whose unaligned 8-voxel cells
+// two lanes share (165 x 92 x 90 at (8, 2, 3) 14.2 against 21.7).  A rule of the geometry
+// only (a 152-SM GPU, 16-byte-aligned gradient), so that a workspace query knows the
+// answer; a tile-config entry that shapes the units' launch keeps them.
 constexpr double kSmallFill = 0.65, kSmallAnyFill = 0.3;
-constexpr int kSmallRows = 48;
+constexpr int kSmallRows = 48, kSmallWork = 60;
+constexpr double kSmallNarrowFill = 0.55, kSmallSplitFill = 0.25;
+constexpr int kSmallSplitRows = 60;
 static bool takes_small(const bsi_geom& g, int n) {
     if (n != 1 || empty_volume(g) || g.dx > kMaxSpecializedDx) return false;
     const bsi_tile_config cfg = lookup_config(g.dx, g.dy, g.dz);
@@ -265,7 +270,12 @@ static bool takes_small(const bsi_geom& g, int n) {
         const int blk = tma_block_bytes(d.dx, d.tma_rows);
         wps = tma_warps_per_cta(blk, tma_default_stages(blk), 0, d.jrows);
     }
+    // the rows that a unit has of the volume; of very few it is as short as a cell's
+    const int planes = imin(d.Z, kMinZChunk * d.dz), yrows = imin(d.Y, d.jrows * d.dy);
+    if (planes * yrows * (d.dx + 4) < kSmallWork && (yrows > 1 || planes < 5)) return false;
     const double fill = (double)d.units / (152.0 * wps);
+    if (d.dx <= 4 && fill >= kSmallNarrowFill) return false;
+    if (d.dx == kMaxSpecializedDx && !tma && fill >= kSmallSplitFill && planes * yrows < kSmallSplitRows) return false;
     const int rows = kMinZChunk * d.dz * d.jrows * d.dy;
     return fill < kSmallAnyFill || (fill < kSmallFill && rows >= kSmallRows);
 }
