@@ -881,9 +881,9 @@ static void check_cells(const RatDesc& d, const CellPlan& c, bool adjoint, Range
     if (!cover) return;
     std::vector<unsigned char> plane((size_t)d.Y * d.Z, 0), written(adjoint ? (size_t)(c.part_floats / 3) : 0, 0);
     for (long long un = 0; un < c.units; ++un) {
-        const CellUnit u = cell_unit(d, c, un);
-        if (u.y1 <= u.y0 || u.y1 - u.y0 > c.ymax || u.z1 < u.z0 || u.z1 - u.z0 > c.zmax || u.y1 > d.Y || u.z1 > d.Z ||
-            u.y0 < 0 || u.z0 < 0)
+        const CellUnit u = cell_unit<true>(d, c, un);
+        if (u.y1 < u.y0 || (u.y1 == u.y0 && c.ysplit == 1) || u.y1 - u.y0 > c.ymax || u.z1 < u.z0 ||
+            u.z1 - u.z0 > c.zmax || u.y1 > d.Y || u.z1 > d.Z || u.y0 < 0 || u.z0 < 0)
             rc.fail("unit rows and planes", u.y1 - u.y0, u.z1 - u.z0);
         if (u.jy + 4 > d.ny || u.kz1 + kHalo > d.nz || u.kz1 <= u.kz0 || u.kz1 - u.kz0 > c.zc) rc.fail("unit cells", u.jy, u.kz0);
         for (int z = u.z0; z < u.z1; ++z) {

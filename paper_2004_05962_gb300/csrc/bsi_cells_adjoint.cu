@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kCellAdjWarps * kLanes, 3)
     float2 W[RUN][2];
     unsigned q = 0;
     for (long long un = (long long)blockIdx.x * wpc + warp; ok_all && un < c.units; un += (long long)gridDim.x * wpc) {
-        const CellUnit u = cell_unit(d, c, un);
+        const CellUnit u = cell_unit<false>(d, c, un);
         __syncwarp();   // the previous unit's weights are read
         unit_weights(d, c, u, yw, zw, lane, &g_err);
         if (u.xs != lxs) {   // warp-uniform: this warp's strip changed

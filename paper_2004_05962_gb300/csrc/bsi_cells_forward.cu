@@ -46,7 +46,9 @@ __device__ __forceinline__ void emit_run(const float2 (&W)[RUN][4], const float 
 
 constexpr int kCellFwdWarps = 4;   // per CTA, three CTAs per SM
 
-template <int RUN, bool WIDE, bool VEC>
+// YSPLIT: units may be parts of y-cells (small volumes; finding one costs 0.5% of 512 x
+// 512 x 300 at spacing 4.7, whose units are whole y-cells).
+template <int RUN, bool WIDE, bool VEC, bool YSPLIT>
 __global__ void __launch_bounds__(kCellFwdWarps * kLanes, 3)
     bsi_cells_forward_kernel(const __grid_constant__ RatDesc d, const __grid_constant__ CellPlan c) {
     extern __shared__ __align__(128) unsigned char csmem[];
@@ -69,7 +71,7 @@ __global__ void __launch_bounds__(kCellFwdWarps * kLanes, 3)
     float2 W[RUN][4];   // each weight twice
     int buf = 0;
     for (long long un = (long long)blockIdx.x * wpc + warp; un < c.units; un += (long long)gridDim.x * wpc) {
-        const CellUnit u = cell_unit(d, c, un);
+        const CellUnit u = cell_unit<YSPLIT>(d, c, un);
         __syncwarp();   // the previous unit's weights are read
         unit_weights(d, c, u, yw, zw, lane, &g_err);
         if (u.xs != lxs) {   // warp-uniform: this warp's strip changed
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(kCellFwdWarps * kLanes, 3)
 
 template <int RUN, bool WIDE, bool VEC>
 static cudaError_t launch_cells_fwd_t(const RatDesc& d, const CellPlan& c, cudaStream_t s) {
-    auto kern = bsi_cells_forward_kernel<RUN, WIDE, VEC>;
+    auto kern = c.ysplit > 1 ? bsi_cells_forward_kernel<RUN, WIDE, VEC, true> : bsi_cells_forward_kernel<RUN, WIDE, VEC, false>;
     const int wpc = imin(kCellFwdWarps, kSmemBudget / c.warp_bytes);
     const int threads = wpc * kLanes, smem = wpc * c.warp_bytes;
     KernelFacts f;

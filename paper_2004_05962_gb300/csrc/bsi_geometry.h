@@ -441,6 +441,7 @@ struct CellPlan {
     int sc, nsx;         // x-cells per strip, strips
     int nc;              // columns a strip touches: sc + 3
     int zc, zsplit;      // z-cells per unit, or (zsplit > 1, zc = 1) units per z-cell
+    int ysplit, nyu;     // units per y-cell (1 in the adjoint), y-units: ncy ysplit
     int nzu;             // z-units: ceil(ncz / zc) or ncz zsplit
     int ymax, zmax;      // most rows of a unit, most planes
     int slot;            // bytes of one staged row (16-byte multiple)
@@ -462,19 +463,20 @@ struct CellUnit {
     int xs, jy, kz0, kz1, z0, z1, y0, y1;
 };
 
+template <bool YSPLIT>
 BSI_HD CellUnit cell_unit(const RatDesc& d, const CellPlan& c, long long un) {
     CellUnit u;
     int zi;
     if (c.units <= 0x7fffffffLL) {   // 32-bit division (64-bit division is a long sequence)
         const unsigned t = (unsigned)un / (unsigned)c.nsx;
         u.xs = (int)((unsigned)un - t * (unsigned)c.nsx);
-        zi = (int)(t / (unsigned)c.ncy);
-        u.jy = (int)(t - (unsigned)zi * (unsigned)c.ncy);
+        zi = (int)(t / (unsigned)c.nyu);
+        u.jy = (int)(t - (unsigned)zi * (unsigned)c.nyu);
     } else {
         u.xs = (int)(un % c.nsx);
         const long long t = un / c.nsx;
-        u.jy = (int)(t % c.ncy);
-        zi = (int)(t / c.ncy);
+        u.jy = (int)(t % c.nyu);
+        zi = (int)(t / c.nyu);
     }
     if (c.zsplit > 1) {
         u.kz0 = zi / c.zsplit;
@@ -490,8 +492,18 @@ BSI_HD CellUnit cell_unit(const RatDesc& d, const CellPlan& c, long long un) {
         u.z0 = a + n * p / c.zsplit;
         u.z1 = a + n * (p + 1) / c.zsplit;
     }
+    int p = 0;   // part of the y-cell
+    if (YSPLIT && c.ysplit > 1) {
+        p = u.jy % c.ysplit;
+        u.jy /= c.ysplit;
+    }
     u.y0 = cell_first(u.jy, d.num[1], d.den[1], d.off[1]);
     u.y1 = imin(d.Y, cell_first(u.jy + 1, d.num[1], d.den[1], d.off[1]));
+    if (YSPLIT && c.ysplit > 1) {
+        const int n = u.y1 - u.y0, a = u.y0;
+        u.y0 = a + n * p / c.ysplit;
+        u.y1 = a + n * (p + 1) / c.ysplit;
+    }
     return u;
 }
 
@@ -542,7 +554,8 @@ constexpr int kCellWarpBudget = (225 * 1024 / kCellWarpsPerSm) & ~127;
 
 // Plan of a volume (a rule of its geometry only, so that a workspace query
 // needs no device).  Adjoint: z-cells per unit, or units per z-cell (forward:
-// one cell, or a part of it), by a cost model of rounds over the warps of a
+// one cell, or a part of it -- where parts of one plane still leave warps idle, of its
+// rows too: forward of 64^3 at 24 12.1 -> 5.4 us, 128^3 at 32 10.3 -> 8.3), by a cost model of rounds over the warps of a
 // 152-SM GPU x rows of a unit, in units of one staged row; a last, partial
 // round costs 0.6 + 0.4 x its fill (a lone warp per scheduler runs faster); a unit costs about kUnitRows rows to start and half
 // a row per plane of partial sums, and a partial sum is written and read once.  Only plans of
@@ -570,15 +583,16 @@ inline CellPlan cell_plan(const RatDesc& d, bool adjoint, bool vec, long long ma
     c.nc = c.sc + kHalo;
     const int vox = imin(d.X, (int)((long long)c.sc * d.num[0] / d.den[0]) + 1);
     c.slot = (12 * vox + 32 + 15) & ~15;
-    c.ymax = widest(1, d.Y);
+    const int yw = widest(1, d.Y);
     c.zmax = kCellRowsMax;
     const int zw = widest(2, d.Z);
     const double rows = (double)d.num[1] / d.den[1], planes = (double)d.num[2] / d.den[2];
     const double slots = 152.0 * kCellWarpsPerSm;
-    c.zc = c.zsplit = 1;
+    c.zc = c.zsplit = c.ysplit = 1;
     auto size = [&](CellPlan& p) {
         p.nzu = p.zsplit > 1 ? p.ncz * p.zsplit : (int)cdiv(p.ncz, p.zc);
-        p.units = (long long)p.nzu * p.ncy * p.nsx;
+        p.nyu = p.ncy * p.ysplit;
+        p.units = (long long)p.nzu * p.nyu * p.nsx;
         p.part_floats = adjoint ? p.units * (p.zc + kHalo) * 4 * 3 * p.nc : 0;
     };
     CellPlan best = c, p = c;
@@ -588,19 +602,25 @@ inline CellPlan cell_plan(const RatDesc& d, bool adjoint, bool vec, long long ma
         p.zc = k < 8 ? 8 - k : 1;
         p.zsplit = k < 8 ? 1 : 1 << (k - 7);
         if (p.zc * zw > kCellRowsMax || p.zsplit > zw) continue;
-        size(p);
-        const bool f = max_floats < 0 || p.part_floats <= max_floats;
-        const double n = p.units / slots, full = (double)(long long)n, part = n - full;
-        const double start = adjoint ? kUnitRows + 0.5 * (p.zc + kHalo) : kUnitRows;
-        const double t = (full + (part > 1e-9 ? 0.6 + 0.4 * part : 0.0)) * (planes * p.zc / p.zsplit * rows + start) +
-                         p.part_floats * 4.0 / (12.0 * vox * slots);
-        if (best_t < 0 || (f && !fits) || (f == fits && (f ? t < best_t : p.part_floats < best.part_floats))) {
-            best = p;
-            best_t = t;
-            fits = f;
+        // parts of y-cells only beside the shortest parts of z-cells
+        const int ymost = !adjoint && 2 * p.zsplit > zw ? yw : 1;
+        for (p.ysplit = 1; p.ysplit <= ymost; p.ysplit *= 2) {
+            size(p);
+            const bool f = max_floats < 0 || p.part_floats <= max_floats;
+            const double n = p.units / slots, full = (double)(long long)n, part = n - full;
+            const double start = adjoint ? kUnitRows + 0.5 * (p.zc + kHalo) : kUnitRows;
+            const double t = (full + (part > 1e-9 ? 0.6 + 0.4 * part : 0.0)) *
+                                 (planes * p.zc / p.zsplit * rows / p.ysplit + start) +
+                             p.part_floats * 4.0 / (12.0 * vox * slots);
+            if (best_t < 0 || (f && !fits) || (f == fits && (f ? t < best_t : p.part_floats < best.part_floats))) {
+                best = p;
+                best_t = t;
+                fits = f;
+            }
         }
     }
     c = best;
+    c.ymax = (int)cdiv(yw, c.ysplit);
     c.zmax = imin(kCellRowsMax, c.zc * zw);
     c.head_bytes = pad128(kCellWeightOff + 16 * (c.ymax + c.zmax));
     int rb = (kCellWarpBudget - c.head_bytes) / (kCellStages * c.slot);

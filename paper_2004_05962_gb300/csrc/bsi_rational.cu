@@ -146,13 +146,26 @@ __global__ void __launch_bounds__(kRatWarps * 32) bsi_rational_window_kernel(con
 // The kernels on cells of any width take x-spacings of 2.5 voxels and more (the
 // windowed kernel's cost is per voxel, theirs per cell; 256 x 256 x 200: at 3
 // 0.048 against 0.064 ms, at 2.33 both 0.090, at 2 0.147 against 0.091), and any
-// on grids wider than the windowed kernel's rings hold.
-static bool rational_takes_cells(const RatDesc& d) {
-    return 2LL * d.num[0] >= 5LL * d.den[0] || d.nx > kRatWindowMaxNx;
+// on grids wider than the windowed kernel's rings hold.  The windowed kernel keeps
+// (us, cells -> windowed)
+// - narrow grids (its line takes a load or two per lane) of at most 10000 rows of 32
+//   voxels, whose time is that of one unit, cells' the longer: 64^3 at 12.5 11.2 ->
+//   5.4, at 4.7 6.7 -> 5.7, 40^3 at 4.7 6.0 -> 4.5;
+// - wide cells of which strips fill less than 60% of their lanes, where the windowed
+//   kernel contracts a grid row for 12 or more output rows: 180 x 70 x 65 at (19, 14,
+//   19) 14.3 -> 6.9, 184 x 271 x 324 at (30, 62, 64) 74.6 -> 59.5.
+static bool rational_takes_cells(const RatDesc& d, const CellPlan& c) {
+    if (d.nx > kRatWindowMaxNx) return true;
+    if (2LL * d.num[0] < 5LL * d.den[0]) return false;
+    if (d.nx <= 24 && d.num[0] > 8 * d.den[0] && d.num[1] >= 12 * d.den[1] &&
+        c.ncx * c.parts < 0.6 * (c.nsx * kLanes))
+        return false;
+    return d.nx > 32 || d.X > 512 || (long long)d.Z * d.Y * cdiv(d.X, 32) > 10000;
 }
 
 cudaError_t launch_forward_rational(const RatDesc& d, cudaStream_t s, LaunchInfo* info) {
-    if (rational_takes_cells(d)) return launch_cells_forward(d, cell_plan(d, false, (reinterpret_cast<uintptr_t>(d.field) & 15) == 0), s);
+    const CellPlan c = cell_plan(d, false, (reinterpret_cast<uintptr_t>(d.field) & 15) == 0);
+    if (rational_takes_cells(d, c)) return launch_cells_forward(d, c, s);
     const bool table = d.X <= kRatTableMaxX;
     const int table_bytes = table ? 20 * d.X : 0;
     const int per_warp = 60 * d.nx;
