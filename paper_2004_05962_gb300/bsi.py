@@ -236,6 +236,13 @@ def _stream(stream, device) -> int:
     return torch.cuda.current_stream(device).cuda_stream
 
 
+def _tensor_stream(stream, device) -> int:
+    """_stream for the device of a CUDA tensor (0.2 us less: a small volume's step takes 26)."""
+    if stream is None and _raw_stream is not None:
+        return _raw_stream(device.index)
+    return _stream(stream, device)
+
+
 def _check(st, where):
     if st:
         detail = library().bsi_last_cuda_error().decode() if st == 8 else ""
@@ -273,7 +280,7 @@ def bsi_field_forward(phi, shape, spacing, out=None, out_dtype=torch.float32, st
     else:
         _need(out, "out", out.dtype, shape + (3,))
     st = library().bsi_field_forward(_geom_ref(g, gst, shape, spacing), phi.data_ptr(), out.data_ptr(),
-                                     _out_dtype_code(out.dtype), _stream(stream, phi.device))
+                                     _out_dtype_code(out.dtype), _tensor_stream(stream, phi.device))
     _check(st, "bsi_field_forward")
     return out
 
@@ -311,7 +318,7 @@ def bsi_field_adjoint(grad_field, spacing, out=None, workspace=None, stream=None
     ws, wsb = _workspace(need, grad_field.device, workspace)
     st = library().bsi_field_adjoint(ref, grad_field.data_ptr(), out.data_ptr(),
                                      ws.data_ptr() if ws is not None else None, wsb,
-                                     _stream(stream, grad_field.device))
+                                     _tensor_stream(stream, grad_field.device))
     _check(st, "bsi_field_adjoint")
     return out
 
@@ -331,7 +338,7 @@ def bsi_field_adjoint_noalloc(grad_field, spacing, out=None, stream=None):
         _need(out, "out", torch.float32, grid)
     ref = _geom_ref(g, gst, shape, spacing)
     st = library().bsi_field_adjoint_noalloc(ref, grad_field.data_ptr(), out.data_ptr(),
-                                             _stream(stream, grad_field.device))
+                                             _tensor_stream(stream, grad_field.device))
     _check(st, "bsi_field_adjoint_noalloc")
     return out
 
@@ -439,7 +446,7 @@ def bsi_field_forward_rational(phi, shape, num, den, off=(0, 0, 0), out=None, st
         _need(out, "out", torch.float32, shape + (3,))
     _check(gst, "bsi_geom_rational_init")
     st = library().bsi_field_forward_rational(ctypes.byref(g), phi.data_ptr(), out.data_ptr(),
-                                              _stream(stream, phi.device))
+                                              _tensor_stream(stream, phi.device))
     _check(st, "bsi_field_forward_rational")
     return out
 
@@ -465,7 +472,7 @@ def bsi_field_adjoint_rational(grad_field, num, den, off=(0, 0, 0), out=None, wo
     ws, wsb = _workspace(nbytes, grad_field.device, workspace)
     st = library().bsi_field_adjoint_rational(ctypes.byref(g), grad_field.data_ptr(), out.data_ptr(),
                                               ws.data_ptr() if ws is not None else None, wsb,
-                                              _stream(stream, grad_field.device))
+                                              _tensor_stream(stream, grad_field.device))
     _check(st, "bsi_field_adjoint_rational")
     return out
 
@@ -484,7 +491,7 @@ def bsi_field_forward_variant(phi, shape, spacing, variant="ttli", out=None, str
     _need(out, "out", torch.float32, shape + (3,))
     g = make_geom(shape, spacing)
     st = library().bsi_field_forward_variant(ctypes.byref(g), phi.data_ptr(), out.data_ptr(), VARIANTS[variant],
-                                             _stream(stream, phi.device))
+                                             _tensor_stream(stream, phi.device))
     _check(st, "bsi_field_forward_variant")
     return out
 
@@ -500,7 +507,7 @@ def bsi_scalar_forward(coeff, shape, spacing, out=None, out_dtype=torch.float32,
     else:
         _need(out, "out", out.dtype, shape)
     st = library().bsi_scalar_forward(_geom_ref(g, gst, shape, spacing), coeff.data_ptr(), out.data_ptr(), _out_dtype_code(out.dtype),
-                                      _stream(stream, coeff.device))
+                                      _tensor_stream(stream, coeff.device))
     _check(st, "bsi_scalar_forward")
     return out
 
@@ -525,7 +532,7 @@ def bsi_resample_forward(phi, shape, spacing, image, out=None, stream=None):
     else:
         _need(out, "out", torch.float32, shape)
     st = library().bsi_resample_forward(_geom_ref(g, gst, shape, spacing), phi.data_ptr(), image.data_ptr(), fX, fY, fZ,
-                                        out.data_ptr(), _stream(stream, phi.device))
+                                        out.data_ptr(), _tensor_stream(stream, phi.device))
     _check(st, "bsi_resample_forward")
     return out
 
@@ -552,7 +559,7 @@ def bsi_resample_backward(phi, shape, spacing, image, grad_warped, out=None, wor
     st = library().bsi_resample_backward(ref, phi.data_ptr(), image.data_ptr(), fX, fY, fZ,
                                          grad_warped.data_ptr(), out.data_ptr(),
                                          ws.data_ptr() if ws is not None else None, wsb,
-                                         _stream(stream, phi.device))
+                                         _tensor_stream(stream, phi.device))
     _check(st, "bsi_resample_backward")
     return out
 
@@ -564,7 +571,7 @@ def bsi_probe_fill(buf: torch.Tensor, value: int = 0, stream=None) -> None:
     if not buf.is_cuda or not buf.is_contiguous():
         raise ValueError("bsi_probe_fill wants a contiguous CUDA tensor")
     st = library().bsi_probe_fill(buf.data_ptr(), buf.numel() * buf.element_size(), value & 0xFFFFFFFF,
-                                  _stream(stream, buf.device))
+                                  _tensor_stream(stream, buf.device))
     _check(st, "bsi_probe_fill")
 
 

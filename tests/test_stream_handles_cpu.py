@@ -38,3 +38,10 @@ def test_without_the_raw_handle_call(current, monkeypatch):
 
 def test_a_given_stream_is_taken(current):
     assert B._stream(_Stream(7), torch.device("cuda", 0)) == 7 and current == []
+
+
+@pytest.mark.parametrize("raw", [lambda index: 40 + index, None], ids=["raw", "no_raw"])
+def test_entry_points_take_the_tensors_stream(current, monkeypatch, raw):
+    monkeypatch.setattr(B, "_raw_stream", raw)
+    assert B._tensor_stream(None, torch.device("cuda", 2)) == (42 if raw else 5)
+    assert B._tensor_stream(_Stream(7), torch.device("cuda", 2)) == 7
