@@ -589,7 +589,7 @@ static void split_tile_planes(InstDesc& d, bool bf16, int c, int rb, int buf_byt
 }
 
 // The resampling's units: strips of resample_strip_tiles tiles (a tile-config entry
-// may fix them), tile-planes split by resample_zparts.
+// may fix them), tile-planes split by resample_zparts or resample_zparts_sm.
 static void plan_resample(InstDesc& d, int buf_bytes, bool grad) {
     if (d.units <= 0) return;
     if (lookup_config(d.dx, d.dy, d.dz).fwd_strip_tiles == 0) d.gcells = resample_strip_tiles(d.ncx, d.dx, grad);
@@ -597,7 +597,11 @@ static void plan_resample(InstDesc& d, int buf_bytes, bool grad) {
     d.units = (long long)d.ncz * d.ncy * d.nxg;
     const int wsm = resample_warp_smem(buf_bytes), wpc = warps_per_cta(wsm, d.warps_req);
     const int ctas = imax(1, imin(3, kTmaSmemBudget / (wpc * wsm + 1024)));
-    d.zparts = resample_zparts(d.units, (long long)device_sms() * ctas * wpc, d.dz, d.dy);
+    const int sms = device_sms();
+    const long long slots = (long long)sms * ctas * wpc;
+    d.zparts = !grad && 2 * d.units >= slots && 4 * d.units < 3 * slots
+                   ? resample_zparts_sm(d.units, sms, wpc, d.dz, d.dy)
+                   : resample_zparts(d.units, slots, d.dz, d.dy);
     d.units *= d.zparts;
 }
 

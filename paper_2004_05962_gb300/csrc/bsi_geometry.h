@@ -205,6 +205,29 @@ inline int resample_zparts(long long units, long long slots, int dz, int dy) {
     return best;
 }
 
+// The same for value mode where whole tile-planes make units for half to three quarters
+// of the warps: two CTAs per SM already run its gathers at their rate, so what counts there
+// is the CTAs of the fullest SM (one alone takes 0.8 of the time of two, each after the third
+// about half), and parts that only fill more warps lose.  Measured (us, the model above -> this):
+// 64 x 290 x 97 at (6, 3, 4) 23.4 -> 16.6, 96 x 167 x 354 at (8, 5, 5) 47.8 -> 39.5; 192 x 192 x
+// 160 at 5 keeps fifths, 55 against 67 whole.  Of 600 random volumes 22 were more than 5% slower
+// than whole, 1.41 times at most; with this 3, 1.19 times.  Below half the model above
+// is as good, from three quarters on better.
+inline int resample_zparts_sm(long long units, int sms, int wpc, int dz, int dy) {
+    int best = 1;
+    double best_t = -1;
+    for (int p = 1; p <= dz; ++p) {
+        const long long k = cdiv(cdiv(units * p, wpc), sms);
+        const double g = k <= 1 ? 0.8 : k == 2 ? 1.0 : 1.5 + 0.48 * (double)(k - 3);
+        const double t = g * ((dz + p - 1) / p * dy + 1.0);
+        if (best_t < 0 || t < best_t) {
+            best = p;
+            best_t = t;
+        }
+    }
+    return best;
+}
+
 template <bool PARTS = true>
 BSI_HD FwdUnit fwd_unit(const InstDesc& d, long long ul) {
     FwdUnit u;
