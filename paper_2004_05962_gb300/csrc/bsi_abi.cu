@@ -224,7 +224,8 @@ static bool takes_wide(const bsi_geom& g, int n) {
 // 44.6 -> 35.1 at (8, 8, 8), 48.1 -> 34.8 at 12 rows per cell, 61 -> 54 at 4; 317 x 203 x
 // 155, 69% and unaligned, 46.4 -> 32.6 and 46.4 -> 33.3, at 4 rows equal; 160 x 400 x 400,
 // 69% and aligned, 72 -> 61 at 64 rows, 57 against 79 at 12; 512 x 512 x 300, 74%, 133
-// against 149.
+// against 149; 136 x 147 x 202 at (8, 3, 5), 17 cells (59%), one more than a strip of
+// cells takes, 13.5 against 19.3.
 // A tile-config entry that shapes the strips' launch keeps them.
 static bool takes_cells_forward(const bsi_geom& g, int n) {
     if (takes_wide(g, n)) return true;
@@ -234,7 +235,7 @@ static bool takes_cells_forward(const bsi_geom& g, int n) {
     const long long ncx = cdiv(g.X, g.dx);
     const double fill = (double)ncx / (double)(cdiv(ncx, kGroupCells) * kGroupCells);
     const int rows = g.dy * g.dz;
-    return (rows >= 12 && fill < (g.X % 4 != 0 ? 0.72 : 0.6)) || (rows >= 48 && fill < 0.72);
+    return (rows >= 12 && fill < (g.X % 4 != 0 ? 0.72 : rows < 16 ? 0.57 : 0.6)) || (rows >= 48 && fill < 0.72);
 }
 
 // Whether the adjoint of one volume takes the kernels on cells of any width though
