@@ -250,12 +250,14 @@ static bool takes_cells_forward(const bsi_geom& g, int n) {
 // 3: 14.1 -> 11.8).  Nor units of few rows in all (882 x 1 x 3 at (3, 2, 6) 6.1 against
 // 8.2; 2920 x 10 x 2 at (1, 8, 7) 7.6 against 14.6), narrow tiles from 55% on (168 x 195
 // x 278 at (4, 7, 6) 32.7 against 45.0) or short units whose unaligned 8-voxel cells
-// two lanes share (165 x 92 x 90 at (8, 2, 3) 14.2 against 21.7).  A rule of the geometry
+// two lanes share (165 x 92 x 90 at (8, 2, 3) 14.2 against 21.7), nor of those any of up to
+// four rows a plane from 45% on (159 x 215 x 397 at (8, 2, 14) 79 against 121, 303 x 148 x 232
+// at (8, 4, 7) 53 against 67).  A rule of the geometry
 // only (a 152-SM GPU, 16-byte-aligned gradient), so that a workspace query knows the
 // answer; a tile-config entry that shapes the units' launch keeps them.
 constexpr double kSmallFill = 0.65, kSmallAnyFill = 0.3;
 constexpr int kSmallRows = 48, kSmallWork = 60;
-constexpr double kSmallNarrowFill = 0.55, kSmallSplitFill = 0.25;
+constexpr double kSmallNarrowFill = 0.55, kSmallSplitFill = 0.25, kSmallSplitShortFill = 0.45;
 constexpr int kSmallSplitRows = 60;
 static bool takes_small(const bsi_geom& g, int n) {
     if (n != 1 || empty_volume(g) || g.dx > kMaxSpecializedDx) return false;
@@ -276,7 +278,9 @@ static bool takes_small(const bsi_geom& g, int n) {
     if (planes * yrows * (d.dx + 4) < kSmallWork && (yrows > 1 || planes < 5)) return false;
     const double fill = (double)d.units / (152.0 * wps);
     if (d.dx <= 4 && fill >= kSmallNarrowFill) return false;
-    if (d.dx == kMaxSpecializedDx && !tma && fill >= kSmallSplitFill && planes * yrows < kSmallSplitRows) return false;
+    if (d.dx == kMaxSpecializedDx && !tma && fill >= kSmallSplitFill &&
+        (planes * yrows < kSmallSplitRows || (yrows <= 4 && fill >= kSmallSplitShortFill)))
+        return false;
     const int rows = kMinZChunk * d.dz * d.jrows * d.dy;
     return fill < kSmallAnyFill || (fill < kSmallFill && rows >= kSmallRows);
 }

@@ -17,7 +17,8 @@ def _tile_planes(shape, spacing):
 
 
 @pytest.mark.parametrize("shape,spacing", [((3, 1, 882), (6, 2, 3)), ((2, 10, 2920), (7, 8, 1)), ((2, 2, 40), (5, 5, 5)),
-                                           ((278, 195, 168), (6, 7, 4)), ((90, 92, 165), (3, 2, 8))])
+                                           ((278, 195, 168), (6, 7, 4)), ((90, 92, 165), (3, 2, 8)),
+                                           ((397, 215, 159), (14, 2, 8)), ((232, 148, 303), (7, 4, 8))])
 def test_tile_planes(shape, spacing):
     assert P.bsi_adjoint_workspace_bytes(shape, spacing) == _tile_planes(shape, spacing)
     n, msg = P.bsi_selfcheck_ranges([shape], [spacing], "adjoint", cover=True)
