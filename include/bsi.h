@@ -115,12 +115,16 @@ size_t bsi_adjoint_workspace_bytes(const bsi_geom* g);
  *                on entry are ignored.  May be NULL when the size is 0.
  * Two kernels: per-warp partial sums over tiles, then a fixed-order reduce.
  * A gradient with X % 4 == 0 at a 16-byte-aligned address and dx <= 8 is read
- * by TMA tensor copies (one per block of rows), any other by one bulk copy per
- * row.  With one tile-row per warp unit both add the same terms in the same
- * order (bitwise equal results); on the tensor-copy path a single volume at
- * y-spacing 4..6 takes units of two tile-rows, which sum in another order
- * (equal to rounding).  The same call on the same input always gives the same
- * bits. */
+ * by TMA tensor copies (one per block of rows), any other in blocks of rows by
+ * one bulk copy per row.  With one tile-row per warp unit both add the same
+ * terms in the same order (bitwise equal results for the same tile-planes per
+ * unit); on the tensor-copy path a single volume at y-spacing 4..6 takes units
+ * of two tile-rows.  One volume too small to fill the GPU with such units, or
+ * with dx > 8 and dy * dz >= 16, takes units of cells instead, split by its
+ * geometry, at some x-spacings also by the gradient's alignment.  Each plan
+ * sums in an order of its own (equal to rounding), so a volume in a batch may
+ * differ in the last bits from the same volume alone.  The same call on the
+ * same input always gives the same bits. */
 bsi_status bsi_field_adjoint(const bsi_geom* g, const float* grad_field, float* grad_phi,
                              void* workspace, size_t workspace_bytes, bsi_stream_t stream);
 

@@ -422,8 +422,9 @@ static void plan_row_stages(Group& g, long long units) {
         }
         return t;
     };
-    // (the heaviest instance's planes have rows to pair)
-    const bool deep = imin(g.inst[0].dy, g.inst[0].Y) > 1 && time(true) <= 1.15 * time(false);
+    // (the stages differ, and the heaviest instance's planes have rows to pair)
+    const bool deep = row_stage_bytes(g.dxmax, true) > row_stage_bytes(g.dxmax, false) &&
+                      imin(g.inst[0].dy, g.inst[0].Y) > 1 && time(true) <= 1.15 * time(false);
     g.row_stage = row_stage_bytes(g.dxmax, deep);
     for (InstDesc& d : g.inst) d.row_block = row_block_rows(d.dx, d.dy, row_stage_bytes(d.dx, deep));
 }

@@ -2,11 +2,13 @@
 // bsi_cells.cuh): partial sums per unit, then one sum per control point.
 //
 // Bound by HBM reads on large volumes (512 x 512 x 300 at spacing 4.7: 0.161 ms
-// alone for 944 MB, 78% of the DRAM peak, 110 M warp instructions; re-reading
+// alone for 944 MB, 78% of the DRAM peak, 100 M warp instructions; re-reading
 // every voxel's weights from shared memory and copying row by row took 240 M and
-// 0.313 ms), by the rows' latency on small ones.  12 warps of 168 registers: the
-// rolling z window (48 sums per lane) and the weights stay in registers.  Two
-// stages of blocks; three (fewer rows each) measured 0.192 against 0.181 ms.
+// 0.313 ms), by the rows' latency on small ones.  12 warps of 168 registers, which
+// hold the rolling z window (48 sums per lane) and the weights; where lanes share
+// a cell, whose rows are summed per tap (48 sums more), 16 to 156 bytes per thread
+// spill.  Two stages of blocks; three (fewer rows each) measured 0.192 against
+// 0.181 ms.
 #include "bsi_cells.cuh"
 
 namespace bsi {

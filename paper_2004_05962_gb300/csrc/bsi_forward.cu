@@ -6,7 +6,8 @@ namespace bsi {
 
 static __device__ unsigned g_err;
 
-// Persistent grid: in round r every warp of the launch takes one unit of the
+// Persistent grid, of the resident CTAs or from eight rounds on a few times as many
+// (launch_fwd_t): in round r every warp of the launch takes one unit of the
 // concatenated unit lists of all instances (slot_unit, CTA-major: the warps of
 // a CTA take neighbouring units).  The per-unit work is near-uniform,
 // so the static assignment balances without an atomic ticket and is

@@ -436,7 +436,7 @@ BSI_HD long long rational_dim(long long N, int num, int den, int off) {
     return N > 0 ? ((N - 1) * den + off) / num + 4 : 4;
 }
 
-// Cells of any width (bsi_cells.cu: non-integer spacing, and integer x-spacings
+// Cells of any width (bsi_cells_forward.cu, bsi_cells_adjoint.cu: non-integer spacing, integer x-spacings
 // above kMaxSpecializedDx as den = 1, off = 0).  A cell of an axis holds the
 // voxels x with floor((x den + off) / num) = its index; its width is the floor
 // or the ceiling of num / den, less at the volume's ends.  A warp takes strips

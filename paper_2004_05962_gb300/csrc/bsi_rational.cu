@@ -8,9 +8,10 @@
 // Two forward kernels and one adjoint:
 // - bsi_cells_forward_kernel / bsi_cells_adjoint_kernel (bsi_cells_forward.cu,
 //   bsi_cells_adjoint.cu): a warp takes a strip of x-cells, its weights in
-//   registers.  Every adjoint, and the forward of x-spacings >= 2.5 voxels.
-// - bsi_rational_window_kernel (narrower x-cells, nx <= 1024): a warp takes a run
-//   of rows of a plane; the lanes contract the grid over z into a ring of four
+//   registers.  Every adjoint, and most forwards of x-spacings >= 2.5 voxels.
+// - bsi_rational_window_kernel (narrower x-cells, small volumes and wide cells that
+//   fill few lanes, nx <= 1024: rational_takes_cells): a warp takes a run of rows
+//   of a plane; the lanes contract the grid over z into a ring of four
 //   grid rows and over y into a line of nx columns in shared memory, then walk
 //   the row voxel by voxel (consecutive lanes, consecutive voxels).
 // Both forwards sum in the same order (z, then y, then x; lowest tap first).
