@@ -290,11 +290,15 @@ def bsi_adjoint_workspace_bytes(shape, spacing) -> int:
     return int(library().bsi_adjoint_workspace_bytes(ctypes.byref(g)))
 
 
-def _workspace(nbytes, device, workspace):
+def _workspace(nbytes, device, workspace, stream=None):
     if nbytes == 0:
         return workspace, 0
     if workspace is None:
         workspace = torch.empty(nbytes, dtype=torch.uint8, device=device)
+        if stream is not None:
+            # freed on return, to the current stream's pool: not to be handed out before ``stream`` is past the call
+            workspace.record_stream(stream if isinstance(stream, torch.cuda.Stream) else
+                                    torch.cuda.ExternalStream(int(stream.cuda_stream), device=device))
     if not workspace.is_cuda or workspace.numel() * workspace.element_size() < nbytes:
         raise ValueError(f"workspace must be a CUDA tensor of at least {nbytes} bytes")
     return workspace, workspace.numel() * workspace.element_size()
@@ -315,7 +319,7 @@ def bsi_field_adjoint(grad_field, spacing, out=None, workspace=None, stream=None
         _need(out, "out", torch.float32, grid)
     ref = _geom_ref(g, gst, shape, spacing)
     need = int(library().bsi_adjoint_workspace_bytes(ref))
-    ws, wsb = _workspace(need, grad_field.device, workspace)
+    ws, wsb = _workspace(need, grad_field.device, workspace, stream)
     st = library().bsi_field_adjoint(ref, grad_field.data_ptr(), out.data_ptr(),
                                      ws.data_ptr() if ws is not None else None, wsb,
                                      _tensor_stream(stream, grad_field.device))
@@ -400,7 +404,7 @@ def bsi_field_adjoint_batched(grads, spacings, outs=None, workspace=None, stream
     arr = _instances(shapes, spacings, grads=grads, dphis=outs)
     dev = grads[0].device if n else torch.device("cuda")
     need = int(library().bsi_batched_adjoint_workspace_bytes(arr, n))
-    ws, wsb = _workspace(need, dev, workspace)
+    ws, wsb = _workspace(need, dev, workspace, stream)
     st = library().bsi_field_adjoint_batched(arr, n, ws.data_ptr() if ws is not None else None, wsb,
                                              _stream(stream, dev))
     _check(st, "bsi_field_adjoint_batched")
@@ -469,7 +473,7 @@ def bsi_field_adjoint_rational(grad_field, num, den, off=(0, 0, 0), out=None, wo
         _need(out, "out", torch.float32, grid)
     _check(gst, "bsi_geom_rational_init")
     nbytes = int(library().bsi_rational_adjoint_workspace_bytes(ctypes.byref(g)))
-    ws, wsb = _workspace(nbytes, grad_field.device, workspace)
+    ws, wsb = _workspace(nbytes, grad_field.device, workspace, stream)
     st = library().bsi_field_adjoint_rational(ctypes.byref(g), grad_field.data_ptr(), out.data_ptr(),
                                               ws.data_ptr() if ws is not None else None, wsb,
                                               _tensor_stream(stream, grad_field.device))
@@ -555,7 +559,7 @@ def bsi_resample_backward(phi, shape, spacing, image, grad_warped, out=None, wor
         _need(out, "out", torch.float32, grid)
     ref = _geom_ref(g, gst, shape, spacing)
     need = int(library().bsi_resample_backward_workspace_bytes(ref))
-    ws, wsb = _workspace(need, phi.device, workspace)
+    ws, wsb = _workspace(need, phi.device, workspace, stream)
     st = library().bsi_resample_backward(ref, phi.data_ptr(), image.data_ptr(), fX, fY, fZ,
                                          grad_warped.data_ptr(), out.data_ptr(),
                                          ws.data_ptr() if ws is not None else None, wsb,
